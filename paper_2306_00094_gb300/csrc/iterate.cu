@@ -965,8 +965,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_refine_update(double *u, const 
 // nPd = ||b||, yw = (r, z), eta = alpha, beta, relres = ||r|| / ||b||, active, iters,
 // n_active, loops.  Every reduction has a fixed order that does not depend on R.
 
-constexpr int CG_WARPS = 8;                   // warps (rows at a time) of a SpMV block
-constexpr int CG_BLOCKS = 8 * 152;            // SpMV blocks (rows strided over them; 64 warps per SM)
+constexpr int CG_UNIT = 32;                   // rows of a SpMV unit
+constexpr int CG_BLOCKS = 6 * 152;            // SpMV blocks (units strided over them)
 constexpr int CG_MAX_R = 32;                  // right-hand sides per CG call
 constexpr int CG_U = 8;                       // nonzeros per SpMV slot loaded at a time
 
@@ -1041,90 +1041,101 @@ __global__ void __launch_bounds__(RED_THREADS) k_cg_init(const double *b, const 
     }
 }
 
-// q = A p (warp per row, double-single products), (p, q) per column, alpha for the active
-// columns.  Lanes are (nonzero slot kg = lane / 8, column cl = lane % 8): the 8 lanes of a slot
-// read one nonzero and the 8 consecutive p entries of its column index (one 32-byte segment
-// of hi and one of lo), the 4 slots take every 4th nonzero of the row; the slots are summed by
-// two shuffles.  Columns come in blocks of 8; each column's arithmetic is the same whatever R.
-__global__ void __launch_bounds__(CG_WARPS * 32) k_cg_spmv(const int64_t *ptr, const int32_t *col, const float *vhi,
-                                                           const float *vlo, const float *ph, const float *pl,
-                                                           const double *p, double *q, int64_t n, int R, double *part,
-                                                           PcgScalars s) {
-    __shared__ double red[CG_WARPS][CG_MAX_R];
+// q = A p (double-single products), (p, q) per column, alpha for the active columns.  A CTA takes
+// units of 32 consecutive rows with 4 CW warps.  Lanes are (nonzero slot kg = lane / 8, position
+// lane % 8): the 4 slots take every 4th nonzero of a row, and the 8 positions are CW columns of
+// 8 / CW rows (CW = R rounded up to a power of two, at most 8; more columns in blocks of 8).  With
+// 8 columns the lanes of a slot read one nonzero and 8 consecutive p entries (one 32-byte segment
+// of hi and one of lo); with one column they work on 8 rows instead of idling.  Bound by the
+// chain ptr -> column -> p entry and the double-single sums (about 12 FP32 operations per
+// nonzero).  On the 6 x 6 table row of the constant kernel (62001 dofs, 25 nonzeros per row, one
+// column): 19.1 us, against 65.8 us with one row per warp and its 8 positions all columns.
+// Each slot's sum runs over its nonzeros in order, the slots are summed by two shuffles, and a
+// unit's 32 products p q by one warp tree per column, so a column's arithmetic is the same
+// whatever R.
+template <int CW>
+__global__ void __launch_bounds__(128 * CW) k_cg_spmv(const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
+                                                      const float *__restrict__ vhi, const float *__restrict__ vlo,
+                                                      const float *__restrict__ ph, const float *__restrict__ pl,
+                                                      const double *__restrict__ p, double *__restrict__ q, int64_t n,
+                                                      int R, double *part, PcgScalars s) {
+    constexpr int NW = 4 * CW, RP = 8 / CW;       // warps, rows of a warp
+    constexpr int NC = CW == 8 ? CG_MAX_R : CW;
+    __shared__ double prods[CG_UNIT][NC + 1], dsum[NC];
     if (*s.n_active == 0) return;
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, kg = lane >> 3, cl = lane & 7;
-    constexpr int NCB = CG_MAX_R / 8;
-    double dacc[NCB];
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, kg = lane >> 3;
+    const int cl = lane & (CW - 1), row = warp * RP + (lane & 7) / CW;
+    if (threadIdx.x < NC) dsum[threadIdx.x] = 0.0;
+    for (int64_t i0 = (int64_t)blockIdx.x * CG_UNIT; i0 < n; i0 += (int64_t)gridDim.x * CG_UNIT) {
+        const int64_t i = i0 + row;
+        const int64_t a = i < n ? ptr[i] : 0, e = i < n ? ptr[i + 1] : 0;
+        for (int c0 = 0; c0 < R; c0 += 8) {
+            const int c = c0 + cl;
+            const bool on = c < R && i < n;
+            float sh = 0.f, sl = 0.f;
+            // CG_U nonzeros per slot at a time: their matrix loads first, then their p gathers,
+            // then the products in order (loads in flight cover the latency)
+            for (int64_t k0 = a + kg; k0 < e; k0 += 4 * CG_U) {
+                float ahv[CG_U], alv[CG_U];
+                int jv[CG_U];
 #pragma unroll
-    for (int cb = 0; cb < NCB; ++cb) dacc[cb] = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * CG_WARPS + warp; i < n; i += (int64_t)gridDim.x * CG_WARPS) {
-        const int64_t a = ptr[i], e = ptr[i + 1];
-#pragma unroll
-        for (int cb = 0; cb < NCB; ++cb) {
-            const int c = cb * 8 + cl;
-            if (cb * 8 < R) {
-                const bool on = c < R;
-                float sh = 0.f, sl = 0.f;
-                // CG_U nonzeros per slot at a time: their matrix loads first, then their p
-                // gathers, then the products in order (loads in flight cover DRAM latency)
-                for (int64_t k0 = a + kg; k0 < e; k0 += 4 * CG_U) {
-                    float ahv[CG_U], alv[CG_U];
-                    int64_t jv[CG_U];
-#pragma unroll
-                    for (int u = 0; u < CG_U; ++u) {
-                        const int64_t k = k0 + 4 * u;
-                        const bool in = k < e;
-                        ahv[u] = in ? __ldg(vhi + k) : 0.f;
-                        alv[u] = in ? __ldg(vlo + k) : 0.f;
-                        jv[u] = in ? (int64_t)__ldg(col + k) : -1;
-                    }
-                    float xhv[CG_U], xlv[CG_U];
-#pragma unroll
-                    for (int u = 0; u < CG_U; ++u) {
-                        const bool in = on && jv[u] >= 0;
-                        xhv[u] = in ? __ldg(ph + jv[u] * R + c) : 0.f;
-                        xlv[u] = in ? __ldg(pl + jv[u] * R + c) : 0.f;
-                    }
-#pragma unroll
-                    for (int u = 0; u < CG_U; ++u) {
-                        if (!on || jv[u] < 0) continue;
-                        const float ah = ahv[u], al = alv[u], xh = xhv[u], xl = xlv[u];
-                        // explicit round-to-nearest intrinsics: no contraction into fma
-                        const float pr = __fmul_rn(ah, xh);
-                        const float pe = fmaf(ah, xh, -pr);              // ah*xh - pr exactly
-                        const float sum = __fadd_rn(sh, pr);             // TwoSum(sh, pr)
-                        const float bb = __fsub_rn(sum, sh);
-                        const float se = __fadd_rn(__fsub_rn(sh, __fsub_rn(sum, bb)), __fsub_rn(pr, bb));
-                        sh = sum;
-                        sl = __fadd_rn(sl, __fadd_rn(se, fmaf(ah, xl, fmaf(al, xh, pe))));
-                    }
+                for (int u = 0; u < CG_U; ++u) {
+                    const int64_t k = k0 + 4 * u;
+                    const bool in = k < e;
+                    ahv[u] = in ? __ldg(vhi + k) : 0.f;
+                    alv[u] = in ? __ldg(vlo + k) : 0.f;
+                    jv[u] = in ? __ldg(col + k) : -1;
                 }
-                double acc = (double)sh + (double)sl;
-                acc += __shfl_xor_sync(0xffffffffu, acc, 8);
-                acc += __shfl_xor_sync(0xffffffffu, acc, 16);
-                if (kg == 0 && on) {
-                    q[i * R + c] = acc;
-                    dacc[cb] += p[i * R + c] * acc;
+                float xhv[CG_U], xlv[CG_U];
+#pragma unroll
+                for (int u = 0; u < CG_U; ++u) {
+                    const bool in = on && jv[u] >= 0;
+                    xhv[u] = in ? __ldg(ph + (int64_t)jv[u] * R + c) : 0.f;
+                    xlv[u] = in ? __ldg(pl + (int64_t)jv[u] * R + c) : 0.f;
+                }
+#pragma unroll
+                for (int u = 0; u < CG_U; ++u) {
+                    if (!on || jv[u] < 0) continue;
+                    const float ah = ahv[u], al = alv[u], xh = xhv[u], xl = xlv[u];
+                    // explicit round-to-nearest intrinsics: no contraction into fma
+                    const float pr = __fmul_rn(ah, xh);
+                    const float pe = fmaf(ah, xh, -pr);              // ah*xh - pr exactly
+                    const float sum = __fadd_rn(sh, pr);             // TwoSum(sh, pr)
+                    const float bb = __fsub_rn(sum, sh);
+                    const float se = __fadd_rn(__fsub_rn(sh, __fsub_rn(sum, bb)), __fsub_rn(pr, bb));
+                    sh = sum;
+                    sl = __fadd_rn(sl, __fadd_rn(se, fmaf(ah, xl, fmaf(al, xh, pe))));
                 }
             }
+            double acc = (double)sh + (double)sl;
+            acc += __shfl_xor_sync(0xffffffffu, acc, 8);
+            acc += __shfl_xor_sync(0xffffffffu, acc, 16);
+            if (kg == 0 && c < R) {
+                prods[row][c] = on ? p[i * R + c] * acc : 0.0;
+                if (on) q[i * R + c] = acc;
+            }
         }
+        __syncthreads();
+        for (int c = warp; c < R; c += NW) {
+            const double v = warp_sum(prods[lane][c]);
+            if (lane == 0) dsum[c] += v;
+        }
+        __syncthreads();
     }
-    // block sums per column, warps in order
-#pragma unroll
-    for (int cb = 0; cb < NCB; ++cb) {
-        const int c = cb * 8 + cl;
-        if (kg == 0 && c < R) red[warp][c] = dacc[cb];
-    }
-    __syncthreads();
-    if (threadIdx.x < R) {
-        double x = 0;
-        for (int w = 0; w < CG_WARPS; ++w) x += red[w][threadIdx.x];
-        part[(int64_t)blockIdx.x * R + threadIdx.x] = x;
-    }
+    if (threadIdx.x < R) part[(int64_t)threadIdx.x * gridDim.x + blockIdx.x] = dsum[threadIdx.x];
     if (!arrive_last(s.counter)) return;
-    for (int cc = warp; cc < R; cc += CG_WARPS) {
+    for (int cc = warp; cc < R; cc += NW) {
+        // the column's block sums, CG_U loads of a lane in flight, added in block order
+        const double *pc = part + (int64_t)cc * gridDim.x;
         double pq = 0;
-        for (int bl = lane; bl < (int)gridDim.x; bl += 32) pq += __ldcg(part + (int64_t)bl * R + cc);
+        for (int b0 = lane; b0 < (int)gridDim.x; b0 += 32 * CG_U) {
+            double v[CG_U];
+#pragma unroll
+            for (int u = 0; u < CG_U; ++u) v[u] = b0 + 32 * u < (int)gridDim.x ? __ldcg(pc + b0 + 32 * u) : 0.0;
+#pragma unroll
+            for (int u = 0; u < CG_U; ++u)
+                if (b0 + 32 * u < (int)gridDim.x) pq += v[u];
+        }
         pq = warp_sum(pq);
         if (lane == 0) s.eta[cc] = (s.active[cc] && pq != 0.0) ? s.yw[cc] / pq : 0.0;
     }
@@ -1915,10 +1926,17 @@ struct Runner {
         const int64_t n = p->n_dofs_total;
         double *u = ws.cg_u.as<double>(), *r = ws.cg_r.as<double>(), *z = ws.cg_z.as<double>(),
                *pv = ws.cg_p.as<double>(), *q = ws.cg_q.as<double>();
-        k_cg_spmv<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(CG_BLOCKS, (n + CG_WARPS - 1) / CG_WARPS)),
-                    CG_WARPS * 32, 0, st>>>(p->d_cg_ptr.as<int64_t>(), p->d_cg_col.as<int32_t>(),
-                                            p->d_cg_vhi.as<float>(), p->d_cg_vlo.as<float>(), ws.cg_ph.as<float>(),
-                                            ws.cg_pl.as<float>(), pv, q, n, R, ws.cg_part.as<double>(), S);
+        const unsigned blocks =
+            (unsigned)std::max<int64_t>(1, std::min<int64_t>(CG_BLOCKS, (n + CG_UNIT - 1) / CG_UNIT));
+        auto spmv = [&](auto kern, int cw) {
+            kern<<<blocks, 128 * cw, 0, st>>>(p->d_cg_ptr.as<int64_t>(), p->d_cg_col.as<int32_t>(),
+                                              p->d_cg_vhi.as<float>(), p->d_cg_vlo.as<float>(), ws.cg_ph.as<float>(),
+                                              ws.cg_pl.as<float>(), pv, q, n, R, ws.cg_part.as<double>(), S);
+        };
+        if (R > 4) spmv(k_cg_spmv<8>, 8);
+        else if (R > 2) spmv(k_cg_spmv<4>, 4);
+        else if (R > 1) spmv(k_cg_spmv<2>, 2);
+        else spmv(k_cg_spmv<1>, 1);
         note_launch();
         auto upd = [&](auto kern) {
             kern<<<red_grid(n, R), RED_THREADS, 0, st>>>(p->d_cg_dinv.as<double>(), pv, q, u, r, z, n, R,
