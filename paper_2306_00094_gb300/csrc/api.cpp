@@ -510,6 +510,12 @@ size_t problem_bytes(const Decomp &d, int64_t n_nodes, int mask) {
     // per scalar subdomain, 3 rigid modes per 2-D peridynamic one)
     const double nco = (double)K * (nc == 1 ? 1 : 3);
     b += 8.0 * nco * nco + ((mask & 2) ? 4.0 * nco * nco : 0.0);
+    // the Lambda-space operators in ELL form (B, B_D and G by rows, their transposes, the places
+    // of the U dofs in the apply inputs)
+    const double nl = (double)d.B_plus.size(), nu = (double)d.u_off[K];
+    double zmax = 1;
+    for (int32_t z : d.node_zeta) zmax = std::max(zmax, (double)z);
+    b += nl * (8 + 16 * zmax + 16 * 2 * (nc == 1 ? 1 : 3) + 2 * 40) + nu * (40 + 16 * zmax);
     return (size_t)(b * 1.05) + (size_t(16) << 20);
 }
 
@@ -569,6 +575,7 @@ nlfeti_status nlfeti_problem_create(nlfeti_ctx *ctx, const nlfeti_mesh *mesh, co
         assemble_all(q.get());
         setup_jump_weights(q.get());
         setup_coarse(q.get());
+        setup_lambda(q.get());
         int flag[4] = {0, 0, 0, 0};
         NLF_CUDA(cudaMemcpy(flag, q->d_flag.p, sizeof(flag), cudaMemcpyDeviceToHost));
         if (flag[1]) fail(NLFETI_E_INVALID, "an interface node belongs to more than 16 subdomains");

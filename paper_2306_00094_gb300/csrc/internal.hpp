@@ -244,6 +244,15 @@ struct nlfeti_problem {
     // B^T entries, U-mode u0, u1), (co_off, n_co), and per B^T entry its Lambda row and the
     // weights sign * Z[u] (3 doubles)
     nlf::DevMem d_gt_range, d_gt_co, d_gt_rows, d_gt_w, d_gt_w32;   // d_gt_w32: FP32 copy
+    // the Lambda-space operators as the cluster kernels read them (lambda_cluster.cuh; lam_ok when
+    // this problem uses them): ELL indices (int32) and values (FP64 and FP32)
+    bool lam_ok = false;
+    int lam_bd_w = 0, lam_bdt_w = 0;                // entries per row of B_D and B_D^T
+    nlf::DevMem d_l_bpm, d_l_bt;                    // rows of B (2 x n_lambda U indices) and of B^T (2 x n_u signed rows)
+    nlf::DevMem d_l_bd_col, d_l_bd_val, d_l_bd_val32, d_l_bdt_row, d_l_bdt_val, d_l_bdt_val32;
+    nlf::DevMem d_l_g_col, d_l_g_val, d_l_g_val32;  // slots of the rows of G (gw x n_lambda)
+    nlf::DevMem d_l_gt_row, d_l_gt_w, d_l_gt_w32;   // B^T entries: Lambda row, weights (3 x entries)
+    nlf::DevMem d_l_u2p, d_l_u2c;                   // per U dof: place in the paired / column apply input (int4)
     nlf::DevMem d_u2sub;                 // per U dof: subdomain (int32)
     nlf::DevMem d_u2v;                   // per U dof: position in the subdomain vectors (int64)
     nlf::DevMem d_vdofs;                 // per subdomain-vector entry: global dof (int32)
@@ -311,6 +320,11 @@ template <typename T> void factor_ops(nlfeti_problem *p, OpPool<T> &pool);
 void build_tiled_half(nlfeti_problem *p);
 void setup_coarse(nlfeti_problem *p);
 void setup_jump_weights(nlfeti_problem *p);
+// the Lambda-space operators in the form the cluster kernels read (after the two above)
+void setup_lambda(nlfeti_problem *p);
+// whether the cluster kernels run this problem: sizes within their limits and clusters of their
+// size schedulable on the device (sets the kernels' attributes)
+bool lambda_clusters_ok(const nlfeti_problem *p, int bd_w);
 void set_error(nlfeti_ctx *c, const std::string &msg);
 // order the library stream after the caller's stream (enter) and the caller's after it (leave)
 void stream_enter(nlfeti_ctx *c);

@@ -23,6 +23,7 @@
 #include <cstring>
 #include <type_traits>
 
+#include <cooperative_groups.h>
 #include <cuda_fp16.h>
 
 #include "solve.hpp"
@@ -906,6 +907,8 @@ __global__ void __launch_bounds__(256) k_coarse_solve(const double *gpart, int p
     a = warp_sum(a);
     if (lane == 0) alpha[(int64_t)i * R + c] = (L)a;
 }
+
+#include "lambda_cluster.cuh"
 
 // refinement update u += du with corr = max |du| / max |u| per column: grid (row blocks,
 // right-hand sides), per-block maxima, the last block to arrive writes corr (maxima do not
@@ -1817,6 +1820,108 @@ struct Runner {
         note_launch();
     }
 
+    // the PCG vectors of the cluster kernels (grouped layout, padded columns): FP32 in lamf; FP64 r
+    // and lambda in lamf, the others in their own buffers
+    template <typename L> LamVecs<L> group_vecs() {
+        const int64_t n = std::max<int64_t>(1, p->n_lambda) * lam_rp(R);
+        if constexpr (std::is_same<L, float>::value) {
+            float *b = ws.lamf.as<float>();
+            return {b, b + n, b + 2 * n, b + 3 * n, b + 4 * n, b + 5 * n, b + 6 * n};
+        } else {
+            double *b = ws.lamf.as<double>();
+            return {b, ws.w.as<double>(), ws.z.as<double>(), ws.y.as<double>(), ws.pv.as<double>(), ws.q.as<double>(),
+                    b + n};
+        }
+    }
+
+    template <typename L> LamArgs<L> lam_args(double tol, int max_it) {
+        LamArgs<L> a{};
+        const LamVecs<L> v = group_vecs<L>();
+        a.bpm = p->d_l_bpm.as<int32_t>();
+        a.bt = p->d_l_bt.as<int32_t>();
+        a.bd_col = p->d_l_bd_col.as<int32_t>();
+        a.bd_val = wt<L>(p->d_l_bd_val, p->d_l_bd_val32);
+        a.bd_w = p->lam_bd_w;
+        a.bdt_row = p->d_l_bdt_row.as<int32_t>();
+        a.bdt_val = wt<L>(p->d_l_bdt_val, p->d_l_bdt_val32);
+        a.bdt_w = p->lam_bdt_w;
+        a.g_col = p->d_l_g_col.as<int32_t>();
+        a.g_val = wt<L>(p->d_l_g_val, p->d_l_g_val32);
+        a.g_w = p->gw;
+        a.gt_row = p->d_l_gt_row.as<int32_t>();
+        a.gt_w = wt<L>(p->d_l_gt_w, p->d_l_gt_w32);
+        a.gt_n = 2 * p->n_lambda;
+        a.gt_range = p->d_gt_range.as<int64_t>();
+        a.gt_co = p->d_gt_co.as<int32_t>();
+        a.nf = p->n_floating;
+        a.ginv = p->d_GtGinv.as<double>();
+        a.ginv32 = p->d_GtGinv32.as<float>();
+        a.nco = p->n_co;
+        a.u2x = (std::is_same<L, float>::value ? p->d_l_u2p : p->d_l_u2c).template as<int4>();
+        a.yU = ws.yU.as<L>();
+        a.r = v.r; a.w = v.w; a.z = v.z; a.y = v.y; a.pv = v.pv; a.q = v.q; a.lam = v.lam;
+        a.x = apply_input<L>(ws);
+        a.nl = (int)p->n_lambda;
+        a.nu = (int)p->n_u;
+        a.R = R;
+        a.s = S;
+        a.tol = tol;
+        a.max_it = max_it;
+        a.limit = max_it + 1;
+        a.cond = cond;
+        return a;
+    }
+
+    template <typename K, typename... A> void lam_launch(K kern, int groups, size_t smem, A... args) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(groups * LC));
+        cfg.blockDim = dim3(LAM_THREADS);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = LC;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        NLF_CUDA(cudaLaunchKernelEx(&cfg, kern, args...));
+        note_launch();
+    }
+
+    // One PCG iteration on the cluster kernels: k_lam_a (which first finishes the iteration before:
+    // q, eta, the updates of p, lambda and r), S apply, k_lam_b, S^+ apply.
+    template <typename T> void iteration_clusters(const OpPool<T> &pool, double tol, int max_it) {
+        using L = T;
+        LamArgs<L> a = lam_args<L>(tol, max_it);
+        const bool mma = use_mma(pool, true);
+        const int4 *u2c = p->d_l_u2c.as<int4>();
+        auto run_cw = [&](auto cw_tag, bool second) {
+            constexpr int CW = decltype(cw_tag)::value;
+            const size_t smem = lam_smem_bytes<L, CW>(p->n_co, p->n_floating);
+            const int groups = lam_rp(R) / CW;
+            if (second) lam_launch(k_lam_b<L, CW>, groups, smem, a);
+            else if (use_cond) lam_launch(k_lam_a<L, CW, 1>, groups, smem, a, u2c);
+            else lam_launch(k_lam_a<L, CW, 0>, groups, smem, a, u2c);
+        };
+        auto go = [&](bool second) {
+            const int cw = lam_cw(R, (int)sizeof(L));
+            if (cw == 1) run_cw(std::integral_constant<int, 1>{}, second);
+            else if (cw == 2) run_cw(std::integral_constant<int, 2>{}, second);
+            else if constexpr (std::is_same<L, float>::value) run_cw(std::integral_constant<int, 4>{}, second);
+        };
+        a.x16 = mma ? ws.xU.as<__half>() : nullptr;
+        go(false);
+        gate = S.n_active;
+        yout_f = std::is_same<L, float>::value ? ws.yU.as<float>() : nullptr;
+        if (mma) symv_mma(pool, ws.yU.as<double>());
+        else symv<T>(pool, 0, apply_input<T>(ws), ws.yU.as<double>(), true);
+        go(true);
+        symv<T>(pool, 1, apply_input<T>(ws), ws.yU.as<double>());
+        yout_f = nullptr;
+        gate = nullptr;
+    }
+
     // One PCG iteration, ten kernels.  The updates of p, lambda and r are stored by the next
     // iteration's k_check_update (kernels before it form p_new and r_new per row), and
     // k_check_update sets the loop condition inside a graph loop.  The Lambda vectors and their
@@ -1825,6 +1930,7 @@ struct Runner {
     // residual corrects what FP32 leaves).  The dot products' tile sums and the PCG scalars are
     // FP64 in both.
     template <typename T> void iteration(const OpPool<T> &pool, double tol, int max_it) {
+        if (p->lam_ok) return iteration_clusters<T>(pool, tol, max_it);
         using L = T;
         const int64_t nl = p->n_lambda, nu = p->n_u;
         const LamVecs<L> v = lam_vecs<L>();
@@ -2070,7 +2176,14 @@ struct Runner {
             dot_final<FIN_NPD>(ws.w.as<double>(), ws.w.as<double>(), nl);
             // p, y and q start at zero and FIN_NPD set eta = beta = 0: the updates the first
             // iteration stores are empty.  The FP32 pass iterates on FP32 copies of r and lambda.
-            if constexpr (std::is_same<T, float>::value) {
+            NLF_CUDA(cudaMemsetAsync(S.loops, 0, sizeof(int), st));
+            if (p->lam_ok) {
+                const LamVecs<T> v = group_vecs<T>();
+                const int64_t n = nl * lam_rp(R);
+                k_group_enter<T><<<grid_for(n), 256, 0, st>>>(ws.r.as<double>(), lam, v.r, v.lam, nl, R,
+                                                              lam_cw(R, (int)sizeof(T)), n);
+                note_launch();
+            } else if constexpr (std::is_same<T, float>::value) {
                 const LamVecs<float> v = lam_vecs<float>();
                 k_lam_enter<<<grid_for(nl * R), 256, 0, st>>>(ws.r.as<double>(), lam, v.r, v.lam, v.pv, v.y, v.q,
                                                               nl * R);
@@ -2086,7 +2199,6 @@ struct Runner {
             if (batched && !p->prof_on && p->opt.graph_loop) {
                 // device-side loop: one launch, one read-back per pass
                 const PcgGraph &g = while_graph<T>(pool, tol, max_it);
-                NLF_CUDA(cudaMemsetAsync(S.loops, 0, sizeof(int), st));
                 NLF_CUDA(cudaGraphLaunch(g.exec, st));
                 loop_body_launches = g.body_launches;   // counted when the scalars are read back
                 done = max_it + 1;                      // skip the chunked loop below
@@ -2121,7 +2233,12 @@ struct Runner {
             }
             if (exec) NLF_CUDA(cudaGraphExecDestroy(exec));
             drop(graph_slots);
-            if constexpr (std::is_same<T, float>::value) {
+            if (p->lam_ok) {
+                const LamVecs<T> v = group_vecs<T>();
+                k_group_exit<T><<<grid_for(nl * R), 256, 0, st>>>(v.lam, v.r, lam, ws.r.as<double>(), nl, R,
+                                                                  lam_cw(R, (int)sizeof(T)));
+                note_launch();
+            } else if constexpr (std::is_same<T, float>::value) {
                 const LamVecs<float> v = lam_vecs<float>();
                 k_lam_exit<<<grid_for(nl * R), 256, 0, st>>>(v.lam, v.r, lam, ws.r.as<double>(), nl * R);
                 note_launch();
@@ -2245,7 +2362,8 @@ void SolveWS::ensure(nlfeti_problem *p, int nR) {
         else m.alloc(c, bytes);
     };
     auto A = [&](DevMem &m, int64_t n) { alloc(m, sizeof(double) * n * R); };
-    A(lam, nl); A(r, nl); A(w, nl); A(z, nl); A(y, nl); A(pv, nl); A(q, nl); A(d, nl); A(cvec, nl); A(dlam, nl);
+    A(lam, nl); A(r, nl); A(d, nl); A(cvec, nl); A(dlam, nl);
+    for (DevMem *m : {&w, &z, &y, &pv, &q}) alloc(*m, sizeof(double) * nl * lam_rp(R));   // with the grouped layout's padding
     A(fU, nu); A(yU, nu); A(uU, nu);
     A(xU, std::max<int64_t>(1, p->n_up));   // apply layout (padding zeroed by the gathers)
     const int R2x = (R + 1) / 2 * 2;
@@ -2367,7 +2485,7 @@ void SolveWS::ensure(nlfeti_problem *p, int nR) {
     alloc(partial, sizeof(double) * std::max(RED_BLOCKS, TILE_MAX_BLOCKS) * R);
     alloc(partial2, sizeof(double) * std::max(RED_BLOCKS, TILE_MAX_BLOCKS) * R);
     alloc(scal, sizeof(double) * R * 7 + sizeof(int) * (2 * R + 8) + sizeof(float) * 3 * R + sizeof(unsigned) * R);
-    alloc(lamf, sizeof(float) * 7 * nl * R);
+    alloc(lamf, sizeof(float) * 7 * nl * lam_rp(R));
     alloc(slot_flags, sizeof(int) * kSlotFlags);
     alloc(frozen, sizeof(int) * R);
     if (alloc_stream) NLF_CUDA(cudaStreamSynchronize(alloc_stream));
@@ -2918,6 +3036,41 @@ int apply_mma_ctas() {
     fit(k_apply_mma<16>, 16); fit(k_apply_mma<32>, 32); fit(k_apply_mma<64>, 64);
     if (per_sm < 1) fail(NLFETI_E_CUDA, "the tensor-core apply does not fit on an SM");
     return sms * per_sm;
+}
+
+bool lambda_clusters_ok(const nlfeti_problem *p, int bd_w) {
+    if (p->n_lambda < 1 || p->n_lambda > LAM_MAX_ROWS || p->n_co > LAM_MAX_CO || bd_w > LAM_MAX_ELL) return false;
+    if (p->n_xp > INT32_MAX || p->n_up > INT32_MAX || p->n_lambda * LAM_MAX_ELL > INT32_MAX) return false;
+    const size_t smem = std::max(lam_smem_bytes<double, 2>(p->n_co, p->n_floating),
+                                 lam_smem_bytes<float, 4>(p->n_co, p->n_floating));
+    if (smem > LAM_MAX_SMEM) return false;
+    bool ok = true;
+    auto fit = [&](auto kern) {
+        NLF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LAM_MAX_SMEM));
+        NLF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(LC);
+        cfg.blockDim = dim3(LAM_THREADS);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = LC;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        ok = ok && n >= 1;
+    };
+    fit(k_lam_a<float, 1, 0>); fit(k_lam_a<float, 2, 0>); fit(k_lam_a<float, 4, 0>);
+    fit(k_lam_a<float, 1, 1>); fit(k_lam_a<float, 2, 1>); fit(k_lam_a<float, 4, 1>);
+    fit(k_lam_a<double, 1, 0>); fit(k_lam_a<double, 2, 0>); fit(k_lam_a<double, 1, 1>); fit(k_lam_a<double, 2, 1>);
+    fit(k_lam_b<float, 1>); fit(k_lam_b<float, 2>); fit(k_lam_b<float, 4>); fit(k_lam_b<double, 1>); fit(k_lam_b<double, 2>);
+    return ok;
 }
 
 int residual_tma_ctas() {

@@ -996,4 +996,87 @@ void setup_jump_weights(nlfeti_problem *p) {
     NLF_CUDA(cudaStreamSynchronize(c->stream));
 }
 
+namespace {
+
+// CSR (row pointers, entries) -> ELL: entry e of row i at e n + i; -1 / 0 past the row's end
+__global__ void k_ell(const int64_t *ptr, const int64_t *idx, const double *val, int64_t n, int w, int32_t *oi, double *ov,
+                      float *ov32) {
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n * w; t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = t % n, q = ptr[i] + t / n;
+        const bool in = q < ptr[i + 1];
+        oi[t] = in ? (int32_t)idx[q] : -1;
+        ov[t] = in ? val[q] : 0.0;
+        ov32[t] = in ? (float)val[q] : 0.0f;
+    }
+}
+
+// the two (at most) signed rows of B^T per U dof, 0 for none (a chain link has one +1 and one -1)
+__global__ void k_ell_bt(const int64_t *ptr, const int64_t *row, int64_t n, int32_t *o) {
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n * 2; t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = t % n, q = ptr[i] + t / n;
+        o[t] = q < ptr[i + 1] ? (int32_t)row[q] : 0;
+    }
+}
+
+__global__ void k_narrow(const int64_t *a, int32_t *o, int64_t n) {
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x)
+        o[t] = (int32_t)a[t];
+}
+
+// n rows of w entries -> w rows of n (indices optional)
+__global__ void k_flip(const int32_t *ai, const double *av, int64_t n, int w, int32_t *oi, double *ov, float *ov32) {
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n * w; t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t s = (t % n) * w + t / n;
+        if (ai) oi[t] = ai[s];
+        ov[t] = av[s];
+        ov32[t] = (float)av[s];
+    }
+}
+
+}  // namespace
+
+void setup_lambda(nlfeti_problem *p) {
+    nlfeti_ctx *c = p->ctx;
+    const int64_t nl = p->n_lambda, nu = p->n_u;
+    int zmax = 0;                    // most copies of a node: entries of a B_D row (one less per B_D^T row)
+    for (int32_t z : p->dec.node_zeta) zmax = std::max(zmax, (int)z);
+    p->lam_ok = lambda_clusters_ok(p, zmax);
+    if (!p->lam_ok) return;
+    p->lam_bd_w = zmax;
+    p->lam_bdt_w = zmax - 1;
+    auto I = [&](DevMem &m, int64_t n) { m.alloc(c, sizeof(int32_t) * std::max<int64_t>(1, n)); return m.as<int32_t>(); };
+    auto V = [&](DevMem &m, int64_t n) { m.alloc(c, sizeof(double) * std::max<int64_t>(1, n)); return m.as<double>(); };
+    auto F = [&](DevMem &m, int64_t n) { m.alloc(c, sizeof(float) * std::max<int64_t>(1, n)); return m.as<float>(); };
+    int32_t *bpm = I(p->d_l_bpm, 2 * nl);
+    k_narrow<<<256, 256, 0, c->stream>>>(p->d_Bp.as<int64_t>(), bpm, nl);
+    k_narrow<<<256, 256, 0, c->stream>>>(p->d_Bm.as<int64_t>(), bpm + nl, nl);
+    k_ell_bt<<<256, 256, 0, c->stream>>>(p->d_Bt_ptr.as<int64_t>(), p->d_Bt_row.as<int64_t>(), nu, I(p->d_l_bt, 2 * nu));
+    const int wd = p->lam_bd_w, wt = p->lam_bdt_w;
+    k_ell<<<256, 256, 0, c->stream>>>(p->d_BD_ptr.as<int64_t>(), p->d_BD_col.as<int64_t>(), p->d_BD_val.as<double>(), nl,
+                                      wd, I(p->d_l_bd_col, nl * wd), V(p->d_l_bd_val, nl * wd),
+                                      F(p->d_l_bd_val32, nl * wd));
+    k_ell<<<256, 256, 0, c->stream>>>(p->d_BDt_ptr.as<int64_t>(), p->d_BDt_row.as<int64_t>(),
+                                      p->d_BDt_val.as<double>(), nu, wt, I(p->d_l_bdt_row, nu * wt),
+                                      V(p->d_l_bdt_val, nu * wt), F(p->d_l_bdt_val32, nu * wt));
+    if (p->n_co > 0) {
+        const int64_t ne = 2 * nl;
+        k_flip<<<256, 256, 0, c->stream>>>(p->d_Gcol.as<int32_t>(), p->d_Gval.as<double>(), nl, p->gw,
+                                           I(p->d_l_g_col, nl * p->gw), V(p->d_l_g_val, nl * p->gw),
+                                           F(p->d_l_g_val32, nl * p->gw));
+        k_narrow<<<256, 256, 0, c->stream>>>(p->d_gt_rows.as<int64_t>(), I(p->d_l_gt_row, ne), ne);
+        k_flip<<<256, 256, 0, c->stream>>>(nullptr, p->d_gt_w.as<double>(), ne, 3, nullptr, V(p->d_l_gt_w, 3 * ne),
+                                           F(p->d_l_gt_w32, 3 * ne));
+    }
+    std::vector<int4> up(nu), uc(nu);
+    for (const SubdomainDesc &d : p->sd)
+        for (int j = 0; j < d.nG; ++j) {
+            up[d.offU + j] = make_int4((int)d.offXp, (int)(2 * ldgx(d.ldG)), (int)paired_col(j), 0);
+            uc[d.offU + j] = make_int4((int)d.offUp, d.ldG, j, d.nG);
+        }
+    upload(c, p->d_l_u2p, up);
+    upload(c, p->d_l_u2c, uc);
+    NLF_CUDA(cudaGetLastError());
+    NLF_CUDA(cudaStreamSynchronize(c->stream));
+}
+
 }  // namespace nlf
