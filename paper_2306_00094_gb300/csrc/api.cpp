@@ -502,7 +502,8 @@ size_t problem_bytes(const Decomp &d, int64_t n_nodes, int mask) {
         if (mask & 2) b += 4.0 * nk * ldM * 3 + 2 * 4.0 * nG * ldG + 2.0 * nG * ldG;   // FP32 + A pairs, S, S^+, FP16 S
     }
     const double scr = sum_nk * 64 * 2 + (double)K * 64 * 64;              // sweep panels
-    if (mask & 1) b += 8.0 * scr;
+    // FP64: the panel and its digits and those of the pivot rows, rows padded to 128
+    if (mask & 1) b += (sum_nk + 128.0 * K) * (512 + 1792 + 8) + (double)K * (32768 + 57344 + 512);
     if (mask & 2) b += 4.0 * scr;
     b += 4.0 * (double)K * (double)n_nodes;                               // node -> subdomain-local maps
     b += 64.0 * sum_nk;                                                   // index maps, vectors, tensor maps

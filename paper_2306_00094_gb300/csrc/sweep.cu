@@ -13,11 +13,12 @@
 // only dense symmetric products with S_k^+ and S_k.
 //
 // Pivot blocks are NB = 64 wide; a step is three launches over all subdomains: invert
-// the pivot block (one CTA per subdomain, in shared memory), form the pivot panels,
-// update all tiles (64x64 CTA tiles, 4x4 register blocking; for the FP32 operators per the
-// factor_tc option 128x128 tiles on the tensor cores, split-TF32, in sweep_tc.cuh: by default
-// in the Omega sweep of A^k, the sweep of the pinned S_k staying on the FP32 pipes).  A non-positive pivot
-// sets the device status word (NLFETI_E_NOT_SPD) instead of trapping.
+// the pivot block (one CTA per subdomain), form the pivot panels, update all tiles.  FP64: on the
+// tensor cores by exact digit products, block upper triangle only (sweep_dg.cuh).  FP32: 64x64 CTA
+// tiles, 4x4 register blocking, or per the factor_tc option 128x128 tiles on the tensor cores,
+// split-TF32, in sweep_tc.cuh: by default in the Omega sweep of A^k, the sweep of the pinned S_k
+// staying on the FP32 pipes.  A non-positive pivot sets the device status word (NLFETI_E_NOT_SPD)
+// instead of trapping.
 #include <algorithm>
 #include <type_traits>
 #include <cmath>
@@ -182,6 +183,7 @@ template <typename T> __global__ void __launch_bounds__(256) k_update(SweepArgs<
 }
 
 #include "sweep_tc.cuh"
+#include "sweep_dg.cuh"
 
 // copy A^k (FP64, ld = nk) into the swept-matrix pool (type T, ld = ldM, zero padding)
 template <typename T> __global__ void k_load_matrix(const double *A, T *Mpool, const SubdomainDesc *sd) {
@@ -436,9 +438,69 @@ template <typename T> __global__ void k_project(T *Sppool, const SubdomainDesc *
     }
 }
 
+// the FP64 sweeps (sweep_dg.cuh): pivots [0, pend[k]) of every matrix
+void run_sweeps_dg(nlfeti_problem *p, double *pool, const std::vector<int64_t> &moff, const std::vector<int32_t> &mdim,
+                   const std::vector<int32_t> &mld, const std::vector<int32_t> &pend, DevMem &scratch) {
+    nlfeti_ctx *c = p->ctx;
+    const int K = p->K;
+    std::vector<int64_t> soff(K);
+    int64_t rows = 0;
+    int maxn = 0, maxp = 0;
+    for (int k = 0; k < K; ++k) {
+        soff[k] = rows;
+        rows += (mdim[k] + DG_TILE - 1) / DG_TILE * DG_TILE;
+        maxn = std::max(maxn, mdim[k]);
+        maxp = std::max(maxp, pend[k]);
+    }
+    if (maxp == 0) return;
+    const size_t tiles = (size_t)(rows / DG_TILE), dbytes = tiles * DG * DG_TBYTES;
+    const size_t need = 2 * dbytes + (size_t)K * DG * (DG_TBYTES / 2) + sizeof(double) * ((size_t)rows * NB + (size_t)K * NB * NB) +
+                        sizeof(int) * (2 * (size_t)rows + 2 * (size_t)K * NB);
+    if (scratch.bytes < need) scratch.alloc(c, need);
+    DevMem d_moff, d_mdim, d_mld, d_pend, d_soff;
+    upload(c, d_moff, moff);
+    upload(c, d_mdim, mdim);
+    upload(c, d_mld, mld);
+    upload(c, d_pend, pend);
+    upload(c, d_soff, soff);
+    DigitArgs a;
+    a.M = pool;
+    a.pan_d = scratch.as<unsigned char>();
+    a.old_d = a.pan_d + dbytes;
+    a.dinv_d = a.old_d + dbytes;
+    a.pan = reinterpret_cast<double *>(a.dinv_d + (size_t)K * DG * (DG_TBYTES / 2));
+    a.dinv = a.pan + rows * NB;
+    a.pan_e = reinterpret_cast<int *>(a.dinv + (size_t)K * NB * NB);
+    a.old_e = a.pan_e + rows;
+    a.dinv_e = a.old_e + rows;
+    a.piv_c = a.dinv_e + (size_t)K * NB;
+    a.moff = d_moff.as<int64_t>();
+    a.mdim = d_mdim.as<int32_t>();
+    a.mld = d_mld.as<int32_t>();
+    a.pend = d_pend.as<int32_t>();
+    a.scr_off = d_soff.as<int64_t>();
+    a.flag = p->d_flag.as<int>();
+    NLF_CUDA(cudaFuncSetAttribute(k_panel_dg, cudaFuncAttributeMaxDynamicSharedMemorySize, DG_SMEM_PAN));
+    NLF_CUDA(cudaFuncSetAttribute(k_update_dg, cudaFuncAttributeMaxDynamicSharedMemorySize, DG_SMEM_UPD));
+    const unsigned nt = (unsigned)((maxn + DG_TILE - 1) / DG_TILE);
+    const unsigned chunks = (nt * (DG_TILE / DG_LB) + DG_CHUNK - 1) / DG_CHUNK;
+    for (int j0 = 0; j0 < maxp; j0 += NB) {
+        a.j0 = j0;
+        k_pivot_dg<<<K, DG_PIV_THREADS, 0, c->stream>>>(a);
+        k_panel_dg<<<dim3(nt, K), DG_PAN_THREADS, DG_SMEM_PAN, c->stream>>>(a);
+        k_update_dg<<<dim3(nt, chunks, K), DG_THREADS, DG_SMEM_UPD, c->stream>>>(a);
+    }
+    const unsigned mt = (unsigned)((maxn + 31) / 32);
+    k_mirror_up<<<dim3(mt, mt, K), 256, 0, c->stream>>>(pool, a.moff, a.mdim, a.mld);
+    NLF_CUDA(cudaGetLastError());
+    NLF_CUDA(cudaStreamSynchronize(c->stream));
+}
+
 template <typename T> void run_sweeps(nlfeti_problem *p, T *pool, const std::vector<int64_t> &moff,
                                       const std::vector<int32_t> &mdim, const std::vector<int32_t> &mld,
                                       const std::vector<int32_t> &pend, DevMem &scratch, bool allow_tc) {
+    if constexpr (std::is_same<T, double>::value) return run_sweeps_dg(p, pool, moff, mdim, mld, pend, scratch);
+    else {
     nlfeti_ctx *c = p->ctx;
     const int K = p->K;
     std::vector<int64_t> soff(K);
@@ -492,6 +554,7 @@ template <typename T> void run_sweeps(nlfeti_problem *p, T *pool, const std::vec
     }
     NLF_CUDA(cudaGetLastError());
     NLF_CUDA(cudaStreamSynchronize(c->stream));
+    }
 }
 
 }  // namespace
