@@ -1282,9 +1282,10 @@ int residual_ds(nlfeti_problem *p, SolveWS &ws, cudaStream_t st, int R, const do
             p->d_rsched_ptr.as<int32_t>(), p->d_rsched_items.as<int32_t>(), ws.ftil.as<double>(),
             p->d_Bt_ptr.as<int64_t>(), p->d_Bt_row.as<int64_t>(), lam, ws.res.as<double>(), R, ws_err(ws, R));
     };
-    if (R >= 8) go(std::integral_constant<int, 8>{});
-    else if (R >= 4) go(std::integral_constant<int, 4>{});
-    else if (R >= 2) go(std::integral_constant<int, 2>{});
+    const int rc = apply_rc(R, 8);
+    if (rc == 8) go(std::integral_constant<int, 8>{});
+    else if (rc == 4) go(std::integral_constant<int, 4>{});
+    else if (rc == 2) go(std::integral_constant<int, 2>{});
     else go(std::integral_constant<int, 1>{});
     return 2;
 }
@@ -1593,7 +1594,9 @@ struct Runner {
         // the autotuner's choice for this operator kind and R (column block, CTAs per SM), else
         // the default block and two CTAs per SM
         const ApplyChoice ch = apply_choice(p, half ? 1 : (sizeof(T) == 8 ? 2 : 0), R);
-        const int rc = ch.rc > 0 ? ch.rc : apply_rc(R, (int)sizeof(T));
+        // (the default shape named by its widest block up to R runs as the default)
+        const bool dflt = ch.rc <= 0 || (ch.rc == apply_rc_below(R, (int)sizeof(T)) && ch.per_sm == 2 && ch.rpw == 4);
+        const int rc = dflt ? apply_rc(R, (int)sizeof(T)) : ch.rc;
         const int ri = rc >= 16 ? 4 : (rc >= 8 ? 3 : (rc >= 4 ? 2 : (rc >= 2 ? 1 : 0)));
         const CUtensorMap *xm = ws.xmaps_rc[sizeof(T) == 8 ? 1 : 0][ri].template as<CUtensorMap>();
         const bool one = ch.rc > 0 && ch.per_sm == 1 && p->sched1_ctas > 0;
@@ -2390,7 +2393,7 @@ void SolveWS::ensure(nlfeti_problem *p, int nR) {
             for (int ri = 0; ri < 5; ++ri) {
                 const int rce = 1 << ri;
                 xmaps_rc[e][ri].release();
-                if (rce > R && rce > 1) continue;
+                if (rce / 2 >= R && rce > 1) continue;      // up to the block that holds all R
                 if (e == 1 && rce > 8) continue;
                 std::vector<CUtensorMap> maps(std::max(1, p->K));
                 std::memset(maps.data(), 0, sizeof(CUtensorMap) * maps.size());
@@ -2620,7 +2623,7 @@ ApplyChoice apply_choice(const nlfeti_problem *p, int kind, int R) {
     auto it = p->tune.find({kind, R});
     if (it != p->tune.end()) return it->second;
     ApplyChoice c;
-    c.rc = apply_rc(R, kind == 2 ? 8 : 4);
+    c.rc = apply_rc_below(R, kind == 2 ? 8 : 4);
     c.per_sm = 2;
     return c;
 }
@@ -2807,7 +2810,7 @@ void autotune_applies(nlfeti_problem *p, int R, const char *cache_path, std::vec
             }
             if (te.rc == -1) {
                 build_tiled_half(p);
-                p->tune[{kind, R}] = ApplyChoice{apply_rc(R, 4), 2, 1};
+                p->tune[{kind, R}] = ApplyChoice{apply_rc_below(R, 4), 2, 1};
             } else {
                 p->tune[{kind, R}] = ApplyChoice{te.rc, te.per_sm, 0, te.rpw};
             }
