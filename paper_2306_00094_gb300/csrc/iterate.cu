@@ -125,6 +125,7 @@ __global__ void k_gather_bd(const int64_t *ptr, const int64_t *col, const L *val
 
 #include "rows.cuh"
 #include "apply_tma.cuh"
+#include "apply_self.cuh"
 #include "apply_mma.cuh"
 #include "residual_tma.cuh"
 #include "residual_csr.cuh"
@@ -1642,14 +1643,33 @@ struct Runner {
                     return;
                   }
                 }
+                // sixteen columns with two CTAs per SM: eight rows per warp and no producer warp (the
+                // default; four rows only when the tuner or the caller names them beside another block)
+                if constexpr (RCT == 16) {
+                    if (dflt || ch.rpw == 8) {
+                        auto self = [&](auto ns_tag, auto mt_tag) {
+                            constexpr int NS = decltype(ns_tag)::value;
+                            using MT = typename decltype(mt_tag)::type;
+                            k_apply_self<16, NS, MT><<<ctas, SELF_THREADS, apply_smem_bytes(16, NS, 256 * (int)sizeof(MT), true),
+                                                       st>>>(
+                                (std::is_same<MT, float>::value ? pool.maps : pool.hmaps).template as<CUtensorMap>(), xm,
+                                std::is_same<MT, float>::value ? use_sp : 0, sd, sptr, sitems, y, R, gate, S.err,
+                                std::is_same<MT, float>::value ? 1.0 : 1.0 / pool.hscale, wait_tries(), p->dbg_withhold,
+                                yout_f);
+                        };
+                        if (half) self(std::integral_constant<int, APPLY_NS_H16>{}, TypeTag<__half>{});
+                        else self(std::integral_constant<int, APPLY_NS>{}, TypeTag<float>{});
+                        return;
+                    }
+                }
                 if (half) {
                     using NSH = std::integral_constant<int, RCT >= 16 ? APPLY_NS_H16 : APPLY_NS_H>;
-                    if constexpr (RCT >= 4)
+                    if constexpr (RCT >= 4 && RCT < 16)
                         if (ch.rpw == 8) return launch(NSH{}, I2{}, I8{}, rc_tag, TypeTag<__half>{});
                     return launch(NSH{}, I2{}, I4{}, rc_tag, TypeTag<__half>{});
                 }
                 using NSF = std::integral_constant<int, APPLY_NS>;
-                if constexpr (RCT >= 4)
+                if constexpr (RCT >= 4 && RCT < 16)
                     if (ch.rpw == 8) return launch(NSF{}, I2{}, I8{}, rc_tag, TypeTag<float>{});
             }
             k_apply_tma<T, RCT><<<ctas, APPLY_THREADS, apply_smem_bytes(RCT, APPLY_NS, APPLY_CB, std::is_same<T, float>::value),
@@ -2994,13 +3014,18 @@ int apply_tma_ctas() {
     };
     fit8(k_apply_tma<float, 4, APPLY_NS, APPLY_MINB, float, ROWS_APPLY, 8>, apply_smem_bytes(4, APPLY_NS));
     fit8(k_apply_tma<float, 8, APPLY_NS, APPLY_MINB, float, ROWS_APPLY, 8>, apply_smem_bytes(8, APPLY_NS));
-    fit8(k_apply_tma<float, 16, APPLY_NS, APPLY_MINB, float, ROWS_APPLY, 8>, apply_smem_bytes(16, APPLY_NS));
     fit8(k_apply_tma<float, 4, APPLY_NS_H, APPLY_MINB, __half, ROWS_APPLY, 8>,
          apply_smem_bytes(4, APPLY_NS_H, APPLY_CB / 2));
     fit8(k_apply_tma<float, 8, APPLY_NS_H, APPLY_MINB, __half, ROWS_APPLY, 8>,
          apply_smem_bytes(8, APPLY_NS_H, APPLY_CB / 2));
-    fit8(k_apply_tma<float, 16, APPLY_NS_H16, APPLY_MINB, __half, ROWS_APPLY, 8>,
-         apply_smem_bytes(16, APPLY_NS_H16, APPLY_CB / 2));
+    auto fit_self = [&](auto kern, int smem) {
+        NLF_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        int b = 0;
+        NLF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, SELF_THREADS, smem));
+        per_sm = std::min(per_sm, b);
+    };
+    fit_self(k_apply_self<16, APPLY_NS, float>, apply_smem_bytes(16, APPLY_NS, APPLY_CB, true));
+    fit_self(k_apply_self<16, APPLY_NS_H16, __half>, apply_smem_bytes(16, APPLY_NS_H16, APPLY_CB / 2, true));
     if (per_sm < 1) fail(NLFETI_E_CUDA, "the interface apply does not fit on an SM");
     // the one-CTA-per-SM variants (schedules of one CTA per SM): their attributes only
     int one = 1 << 20;
