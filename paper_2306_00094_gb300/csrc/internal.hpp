@@ -244,8 +244,8 @@ struct nlfeti_problem {
     // B^T entries, U-mode u0, u1), (co_off, n_co), and per B^T entry its Lambda row and the
     // weights sign * Z[u] (3 doubles)
     nlf::DevMem d_gt_range, d_gt_co, d_gt_rows, d_gt_w, d_gt_w32;   // d_gt_w32: FP32 copy
-    // the Lambda-space operators as the cluster kernels read them (lambda_cluster.cuh; lam_ok when
-    // this problem uses them): ELL indices (int32) and values (FP64 and FP32)
+    // the Lambda-space operators as the PCG iterations read them (lambda_cluster.cuh when lam_ok, else
+    // lambda_rows.cuh): ELL indices (int32) and values (FP64 and FP32)
     bool lam_ok = false;
     int lam_bd_w = 0, lam_bdt_w = 0;                // entries per row of B_D and B_D^T
     nlf::DevMem d_l_bpm, d_l_bt;                    // rows of B (2 x n_lambda U indices) and of B^T (2 x n_u signed rows)
@@ -320,7 +320,7 @@ template <typename T> void factor_ops(nlfeti_problem *p, OpPool<T> &pool);
 void build_tiled_half(nlfeti_problem *p);
 void setup_coarse(nlfeti_problem *p);
 void setup_jump_weights(nlfeti_problem *p);
-// the Lambda-space operators in the form the cluster kernels read (after the two above)
+// the Lambda-space operators in the form the PCG iterations read (after the two above)
 void setup_lambda(nlfeti_problem *p);
 // whether the cluster kernels run this problem: sizes within their limits and clusters of their
 // size schedulable on the device (sets the kernels' attributes)

@@ -321,156 +321,6 @@ __device__ __forceinline__ bool arrive_last(unsigned *counter) {
     return last;
 }
 
-// Coalesced reductions over Lambda with R interleaved right-hand sides (entry (i, c) at
-// i R + c).  The rows are cut into tiles of RT = 8 rows; block b owns the contiguous tiles
-// [b tpb, (b + 1) tpb) (tpb from n and the grid only).  A (tile, chunk of cw columns) unit
-// takes 4 cw lanes: lane (h, j), h = 0..3, adds rows h and h + 4 of column c0 + j, and the
-// four lanes of a column are added as ((h0 + h2) + (h1 + h3)).  The block adds its tile sums
-// per column in tile order (rounds of up to RSMEM / R tiles through shared memory), and
-// finish_scalars adds the blocks' partials in block order.  cw = min(8, R rounded up to a
-// power of two) and the round size only decide which lanes run a unit and when, never the
-// order of the additions, so every column is summed in the same order whatever the batch it
-// is part of; the lanes of a unit read 4 rows x cw consecutive columns per step, and each lane
-// has two rows in flight.  f(i, c) is called once per entry (i < n, c < R) and returns its
-// addend; a unit's sum is formed in the addends' type (FP32 in the FP32 pass), the tile sums
-// onward in FP64.  The block partials are stored column by column (partial[c * blocks + b]), so that the
-// last block reads each column's partials as whole lines (measured: the finish of 608 blocks x 16
-// columns took 10 us with the partials row by row, 6 us column by column).
-constexpr int RT = 8;
-constexpr int RSMEM = 2048;             // doubles of tile sums per round (16 KB)
-constexpr int TILE_THREADS = 1024;      // threads of a tile-reduction block (one block per SM)
-constexpr int RCOLS = TILE_THREADS;     // columns per pass (one accumulating thread each)
-
-// one 1024-thread CTA per SM: the warps of four 256-thread CTAs, a quarter of the partials for
-// the last block to add (measured: the finish with 608 blocks took about 6 us of each fused
-// reduction, its loads in several dependent rounds)
-constexpr int TILE_MAX_BLOCKS = 152;
-inline int tile_blocks(int64_t n) {
-    const int64_t nt = (n + RT - 1) / RT;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(TILE_MAX_BLOCKS, (nt + 1) / 2));
-}
-
-template <typename F>
-__device__ __forceinline__ void tile_reduce(int64_t n, int R, double *partial, F &&f) {
-    using A = decltype(f(int64_t(0), 0));   // the addends' type: the four-lane unit sums in it
-    __shared__ double ts[RSMEM];
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    const int64_t ntiles = (n + RT - 1) / RT;
-    const int64_t tpb = (ntiles + gridDim.x - 1) / gridDim.x;
-    const int64_t t0 = (int64_t)blockIdx.x * tpb, t1 = min(ntiles, t0 + tpb);
-    const int cw = R >= 5 ? 8 : (R >= 3 ? 4 : (R == 2 ? 2 : 1));
-    const int ulanes = 4 * cw, upw = 32 / ulanes;
-    const int ju = lane / ulanes, jl = lane % ulanes, h = jl / cw, cj = jl % cw;
-    for (int cc0 = 0; cc0 < R; cc0 += RCOLS) {
-        const int ncol = min(RCOLS, R - cc0);
-        const int nchunk = (ncol + cw - 1) / cw;
-        const int rtiles = max(1, min(256, RSMEM / ncol));
-        double acc = 0;
-        for (int64_t tb = t0; tb < t1; tb += rtiles) {
-            const int ntl = (int)min((int64_t)rtiles, t1 - tb);
-            const int units = ntl * nchunk;
-            for (int ub = warp * upw; ub < units; ub += (TILE_THREADS / 32) * upw) {
-                const int u = ub + ju;
-                const int tl = u / nchunk, cl = (u % nchunk) * cw + cj;
-                const bool ok = u < units && cl < ncol;
-                A v = 0;
-                if (ok) {
-                    const int64_t i0 = (tb + tl) * RT + h;
-                    if (i0 < n) v += f(i0, cc0 + cl);
-                    if (i0 + 4 < n) v += f(i0 + 4, cc0 + cl);
-                }
-                v += __shfl_down_sync(0xffffffffu, v, 2 * cw);
-                v += __shfl_down_sync(0xffffffffu, v, cw);
-                if (ok && h == 0) ts[tl * ncol + cl] = (double)v;
-            }
-            __syncthreads();
-            if (threadIdx.x < ncol)
-                for (int tl = 0; tl < ntl; ++tl) acc += ts[tl * ncol + threadIdx.x];
-            __syncthreads();
-        }
-        if (threadIdx.x < ncol) partial[(int64_t)(cc0 + threadIdx.x) * gridDim.x + blockIdx.x] = acc;
-    }
-}
-
-// last block: column totals over the nb row-block partials (warp per column, fixed order)
-// and the PCG scalar update:
-//   NPD:   ||P d|| and the initial state;      CHECK: ||w|| and the active mask;
-//   BETA:  (y,w) and beta = (y,w)/(y,w)_old;    ETA:   (p,q) and eta = (y,w)/(p,q).
-constexpr int FIN_GROUP = 8;            // partials per lane loaded together by the last block
-template <int MODE>
-__device__ void finish_scalars(const double *partial, int nb, int R, PcgScalars s, double tol, int max_it) {
-    __shared__ int n_act;
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    if (threadIdx.x == 0) n_act = 0;
-    __syncthreads();
-    for (int c = warp; c < R; c += TILE_THREADS / 32) {
-        // the column's nb partials are contiguous: each group of loads reads whole lines, with
-        // FIN_GROUP loads of a lane in flight together, added in block order
-        const double *pc = partial + (int64_t)c * nb;
-        double v = 0;
-        for (int b0 = lane; b0 < nb; b0 += 32 * FIN_GROUP) {
-            double pv[FIN_GROUP];
-#pragma unroll
-            for (int m = 0; m < FIN_GROUP; ++m) pv[m] = b0 + 32 * m < nb ? __ldcg(pc + b0 + 32 * m) : 0.0;
-#pragma unroll
-            for (int m = 0; m < FIN_GROUP; ++m)
-                if (b0 + 32 * m < nb) v += pv[m];
-        }
-        v = warp_sum(v);
-        if (lane == 0) {
-            if (MODE == FIN_NPD) {
-                s.nPd[c] = sqrt(v);
-                s.active[c] = 1;
-                s.iters[c] = 0;
-                s.yw_old[c] = 1.0;
-                s.relres[c] = 1.0;
-                s.eta[c] = 0.0;
-                s.beta[c] = 0.0;
-                s.eta_f[c] = 0.0f;
-                s.beta_f[c] = 0.0f;
-                s.xscale_f[c] = 1.0f;
-            } else if (MODE == FIN_CHECK) {
-                const double nw = sqrt(v), ref = s.nPd[c];
-                // a power of two that FP32 holds too (the FP32 pass scales with the same factor)
-                const double xs = (nw > 0.0 && nw < INFINITY) ? ldexp(1.0, max(-126, min(126, -ilogb(nw)))) : 1.0;
-                s.xscale[c] = xs;
-                s.xscale_f[c] = (float)xs;
-                int act = s.active[c];
-                if (act) s.relres[c] = ref > 0 ? nw / ref : 0.0;
-                if (act && (nw <= tol * ref || s.iters[c] >= max_it)) act = 0;
-                s.active[c] = act;
-                if (act) atomicAdd(&n_act, 1);
-            } else if (MODE == FIN_BETA) {
-                s.yw[c] = v;
-                const double b = (s.iters[c] == 0 || s.yw_old[c] == 0.0) ? 0.0 : v / s.yw_old[c];
-                s.beta[c] = b;
-                s.beta_f[c] = (float)b;
-            } else {
-                const bool act = s.active[c] != 0;
-                const double e = (act && v != 0.0) ? s.yw[c] / v : 0.0;
-                s.eta[c] = e;
-                s.eta_f[c] = (float)e;
-                if (act) { s.yw_old[c] = s.yw[c]; s.iters[c] += 1; }
-            }
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        if (MODE == FIN_NPD) *s.n_active = R;
-        if (MODE == FIN_CHECK) *s.n_active = n_act;
-        *s.counter = 0u;
-    }
-}
-
-// (a, b) per column with the scalar update of MODE (grid tile_blocks(n))
-template <int MODE>
-__global__ void __launch_bounds__(TILE_THREADS) k_dot_final(const double *__restrict__ a, const double *__restrict__ b,
-                                                            int64_t n, int R, double *partial, PcgScalars s, double tol,
-                                                            int max_it) {
-    tile_reduce(n, R, partial, [&](int64_t i, int c) { return a[i * R + c] * b[i * R + c]; });
-    if (arrive_last(s.counter)) finish_scalars<MODE>(partial, gridDim.x, R, s, tol, max_it);
-}
-
 // The updates of p, lambda and r are stored one iteration late, by the kernel that starts the
 // next iteration; until then the kernels that read p_new or r_new form them per row with these
 // (the same bits everywhere):
@@ -481,87 +331,6 @@ template <typename L> __device__ __forceinline__ L p_next(L p, L y, L beta, bool
     return active ? fma_l(beta, p, y) : p;
 }
 template <typename L> __device__ __forceinline__ L r_next(L r, L q, L eta) { return fma_l(-eta, q, r); }
-
-// out = P v = v - G alpha (alpha from k_proj_g; NULL when there is no coarse space), with the
-// dot product of MODE: CHECK (out, out), BETA (out, other).  Grid tile_blocks(nl).
-template <int MODE, typename L>
-__global__ void __launch_bounds__(TILE_THREADS) k_project_dot(const int32_t *__restrict__ gcol,
-                                                              const L *__restrict__ gval, int gw,
-                                                              const L *__restrict__ alpha,
-                                                              const L *__restrict__ v,
-                                                              const L *__restrict__ other,
-                                                              L *__restrict__ out, int64_t nl, int R,
-                                                              double *partial, PcgScalars s, double tol, int max_it) {
-    tile_reduce(nl, R, partial, [&](int64_t i, int c) {
-        const int64_t t = i * R + c;
-        L x = v[t];
-        if (alpha) x += -g_alpha(gcol, gval, gw, alpha, i, c, R);
-        out[t] = x;
-        return x * (MODE == FIN_CHECK ? x : other[t]);
-    });
-    if (arrive_last(s.counter)) finish_scalars<MODE>(partial, gridDim.x, R, s, tol, max_it);
-}
-
-// q = B y_U with (p_new, q) and the ETA update (p_new formed per row, stored by the next
-// iteration's k_check_update).  Grid tile_blocks(nl).
-template <typename L>
-__global__ void __launch_bounds__(TILE_THREADS) k_gather_b_eta(const int64_t *__restrict__ Bp,
-                                                               const int64_t *__restrict__ Bm,
-                                                               const L *__restrict__ yU,
-                                                               const L *__restrict__ pv,
-                                                               const L *__restrict__ y, L *__restrict__ q,
-                                                               int64_t nl, int R, double *partial, PcgScalars s) {
-    const L *beta = beta_of<L>(s);
-    tile_reduce(nl, R, partial, [&](int64_t i, int c) {
-        const int64_t t = i * R + c;
-        const L x = yU[Bp[i] * R + c] - yU[Bm[i] * R + c];
-        q[t] = x;
-        return p_next(pv[t], y[t], beta[c], s.active[c] != 0) * x;
-    });
-    if (arrive_last(s.counter)) finish_scalars<FIN_ETA>(partial, gridDim.x, R, s, 0.0, 0);
-}
-
-// Start of a PCG iteration (after k_proj_g formed alpha from G^T r_new): the previous
-// iteration's updates p = p_new, lambda += eta p, r = r_new, then w = P r = r - G alpha,
-// (w, w) and the stop test.  The active flags read here are those p_new was formed with: the
-// last block changes them only after every block has arrived.  COND: the last block also
-// counts the iteration and sets the condition of the WHILE loop (continue while a
-// right-hand side is active and fewer than limit iterations have run, so the loop ends
-// whatever the scalars hold); a separate instantiation, as profilers skip kernels that set
-// graph conditions.
-template <int COND, typename L>
-__global__ void __launch_bounds__(TILE_THREADS) k_check_update(const int32_t *__restrict__ gcol,
-                                                               const L *__restrict__ gval, int gw,
-                                                               const L *__restrict__ alpha,
-                                                               const L *__restrict__ y, L *__restrict__ pv,
-                                                               L *__restrict__ lam, L *__restrict__ r,
-                                                               const L *__restrict__ q, L *__restrict__ w,
-                                                               int64_t nl, int R, double *partial, PcgScalars s,
-                                                               double tol, int max_it, cudaGraphConditionalHandle cond,
-                                                               int limit) {
-    const L *eta = eta_of<L>(s), *beta = beta_of<L>(s);
-    tile_reduce(nl, R, partial, [&](int64_t i, int c) {
-        const int64_t t = i * R + c;
-        const L e = eta[c];
-        const L pn = p_next(pv[t], y[t], beta[c], s.active[c] != 0);
-        pv[t] = pn;
-        lam[t] = fma_l(e, pn, lam[t]);
-        const L rn = r_next(r[t], q[t], e);
-        r[t] = rn;
-        L x = rn;
-        if (alpha) x += -g_alpha(gcol, gval, gw, alpha, i, c, R);
-        w[t] = x;
-        return x * x;
-    });
-    if (arrive_last(s.counter)) {
-        finish_scalars<FIN_CHECK>(partial, gridDim.x, R, s, tol, max_it);
-        if (COND && threadIdx.x == 0) {
-            const int l = *s.loops + 1;
-            *s.loops = l;
-            cudaGraphSetConditional(cond, (*s.n_active > 0 && l < limit) ? 1u : 0u);
-        }
-    }
-}
 
 // Entry of the FP32 pass's iterations: r and lambda rounded to FP32, p, y and q zero; and its
 // exit: lambda and r back in FP64.  n = n_lambda R entries.
@@ -579,28 +348,6 @@ __global__ void k_lam_exit(const float *lf, const float *rf, double *lam, double
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
         lam[t] = (double)lf[t];
         r[t] = (double)rf[t];
-    }
-}
-
-// x (apply layout) = B^T p_new (B^T rows signed r+1 / -(r+1)), p_new formed per row: the input
-// of the S^+ apply of a PCG iteration
-template <typename T, typename L>
-__global__ void k_gather_apply_p(const int64_t *ptr, const int64_t *row, const L *pv, const L *y, const L *beta,
-                                 const int *active, T *x, const SubdomainDesc *sd, const int32_t *u2sub, int64_t nu,
-                                 int R, const int *gate) {
-    if (gate && *gate == 0) return;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nu * R; t += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(t / nu);
-        const int64_t u = t % nu;
-        const bool act = active[c] != 0;
-        const L be = beta[c];
-        L s = 0;
-        for (int64_t q = ptr[u]; q < ptr[u + 1]; ++q) {
-            const int64_t r = row[q], i = r > 0 ? r - 1 : -r - 1;
-            const L pn = p_next(pv[i * R + c], y[i * R + c], be, act);
-            s += r > 0 ? pn : -pn;
-        }
-        apply_store<T>(x, sd, u2sub, u, c, R, (T)s);
     }
 }
 
@@ -631,28 +378,6 @@ __device__ __forceinline__ void gather_x_block(T *x, const SubdomainDesc *sd, co
         const int c = t / nuu, ul = t % nuu;
         apply_store<T>(x, sd, u2sub, u0 + ul, c, R, (T)gx_sm[c * GX_U + ul]);
     }
-}
-
-// x = B^T p_new (as k_gather_apply_p)
-template <typename T, typename L>
-__global__ void __launch_bounds__(256) k_gather_apply_p_t(const int64_t *__restrict__ ptr,
-                                                          const int64_t *__restrict__ row,
-                                                          const L *__restrict__ pv, const L *__restrict__ y,
-                                                          const L *beta, const int *active, T *x,
-                                                          const SubdomainDesc *sd, const int32_t *u2sub, int64_t nu,
-                                                          int R, const int *gate) {
-    if (gate && *gate == 0) return;
-    gather_x_block<T>(x, sd, u2sub, nu, R, [&](int64_t u, int c) {
-        const bool act = active[c] != 0;
-        const L be = beta[c];
-        L s = 0;
-        for (int64_t q = ptr[u]; q < ptr[u + 1]; ++q) {
-            const int64_t r = row[q], i = r > 0 ? r - 1 : -r - 1;
-            const L pn = p_next(pv[i * R + c], y[i * R + c], be, act);
-            s += r > 0 ? pn : -pn;
-        }
-        return s;
-    });
 }
 
 // x = B^T v, or B_D^T v when val is given (as k_gather_apply)
@@ -690,22 +415,6 @@ __device__ __forceinline__ void store_f16(__half *x, const SubdomainDesc *sd, co
     x[col + j] = to_half(v);
     if (j == d.nG - 1)
         for (int q = d.nG; q < d.ldG; ++q) x[col + q] = __float2half(0.0f);
-}
-
-// x (apply layout, FP16) = xscale B_D^T v for the tensor-core preconditioner apply (the sums
-// of k_gather_apply in the type of the Lambda vectors, scaled exactly, rounded once)
-template <typename L>
-__global__ void k_gather_apply_f16(const int64_t *ptr, const int64_t *row, const L *val, const L *v, const L *xscale,
-                                   __half *x, const SubdomainDesc *sd, const int32_t *u2sub, int64_t nu, int R,
-                                   const int *gate) {
-    if (gate && *gate == 0) return;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nu * R; t += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(t / nu);
-        const int64_t u = t % nu;
-        L s = 0;
-        for (int64_t q = ptr[u]; q < ptr[u + 1]; ++q) s += val[q] * v[row[q] * R + c];
-        store_f16(x, sd, u2sub, u, c, R, s * xscale[c]);
-    }
 }
 
 // xscale[c] = 2^-floor(log2 max_u |v[u][c]|) (1 for a zero column); grid R blocks
@@ -752,25 +461,19 @@ __global__ void k_stage_rows_x(const double *xa, const double *xb, const Subdoma
     }
 }
 
-// alpha = (G^T G)^-1 G^T v.  G^T v is gathered from flat entry lists per floating subdomain
-// f: for v on Lambda, entry e of B^T restricted to Gamma_f is (Lambda row rows[e], weights
-// w[e][q] = sign(e) Z[u(e)][q]); for v on U, the entries are the U dofs of Gamma_f with
-// weights Z.  Grid (floating subdomains, psplit slices of the entry range, right-hand sides):
-// block (f, j, c) sums slice j into gpart.  Small coarse spaces (fused): the last block to
-// arrive adds the slices in order (into shared memory when they fit, else gsum) and applies
-// (G^T G)^-1.  Large ones: k_coarse_solve does that over many CTAs (FP64 runs at a small
-// fraction of the FP32 rate here, so one CTA would take ~100 us for n_co = 108 and 16
-// right-hand sides).  In the FP32 pass the large ones are fused per column instead (fused = 2,
-// one slice): the last of a column's blocks to arrive applies the FP32 copy of (G^T G)^-1,
-// stored transposed (GtGinv32[j n_co + i] = (G^T G)^-1[i][j]), to that column, thread i
-// summing over j in ascending order (n_co^2 FP32 FMAs per column: a few thousand cycles of
-// one SM).  psplit and the choice depend on the problem only, so every column is summed in the
-// same order whatever batch it is part of.
-// v_mode: PG_U v on U; PG_LAM v on Lambda; PG_LAM_R r_new = r - eta q on Lambda (v = r)
+// alpha = (G^T G)^-1 G^T v of a sweep's set-up and exit (FP64; the iterations use k_proj_v).  G^T v is
+// gathered from flat entry lists per floating subdomain f: for v on Lambda, entry e of B^T restricted
+// to Gamma_f is (Lambda row rows[e], weights w[e][q] = sign(e) Z[u(e)][q]); for v on U, the entries are
+// the U dofs of Gamma_f with weights Z.  Grid (floating subdomains, psplit slices of the entry range,
+// right-hand sides): block (f, j, c) sums slice j into gpart.  Small coarse spaces (fused): the last
+// block to arrive adds the slices in order (into shared memory when they fit, else gsum) and applies
+// (G^T G)^-1.  Large ones: k_coarse_solve does that over many CTAs.  psplit and the choice depend on
+// the problem only, so every column is summed in the same order whatever batch it is part of.
+// v_mode: PG_U v on U; PG_LAM v on Lambda
 constexpr int PSPLIT = 8;
 constexpr int kCoarseFusedMax = 16;     // n_co up to which the last block of k_proj_g solves
-constexpr int kCoarseColMax = 2048;     // n_co up to which the FP32 pass fuses per column
-enum { PG_U = 0, PG_LAM = 1, PG_LAM_R = 2 };
+constexpr int kCoarseColMax = 2048;     // n_co up to which the FP32 iterations fuse per column group
+enum { PG_U = 0, PG_LAM = 1 };
 
 // true in the last of column c's blocks (gridDim.x gridDim.y of them) to arrive
 __device__ __forceinline__ bool arrive_last_col(unsigned *counters, int c) {
@@ -783,31 +486,27 @@ __device__ __forceinline__ bool arrive_last_col(unsigned *counters, int c) {
     return last;
 }
 
-// L: the type of v, q, the weights, the per-block sums and alpha (FP32 in the FP32 pass, with
-// FP32 copies of the weights); the slices' sums and (G^T G)^-1 are FP64 (but for fused = 2).
-template <int VMODE, typename L>
+template <int VMODE>
 __global__ void __launch_bounds__(256) k_proj_g(const int64_t *range, const int32_t *fco, const int64_t *rows,
-                                                const L *w, const L *v, const L *q, const L *eta, double *gpart,
-                                                double *gsum, const double *GtGinv, int nco, L *alpha, int R,
-                                                unsigned *counter, int psplit, int fused,
-                                                const float *GtGinv32 = nullptr, unsigned *colcnt = nullptr) {
+                                                const double *w, const double *v, double *gpart, double *gsum,
+                                                const double *GtGinv, int nco, double *alpha, int R,
+                                                unsigned *counter, int psplit, int fused) {
     constexpr int lam_mode = VMODE != PG_U;
     extern __shared__ double gs_dyn[];
-    __shared__ L red[8][3];
+    __shared__ double red[8][3];
     const int f = blockIdx.x, c = blockIdx.z;
     const int64_t e0 = range[4 * f + (lam_mode ? 0 : 2)], e1 = range[4 * f + (lam_mode ? 1 : 3)];
     const int co_off = fco[2 * f], nq = fco[2 * f + 1];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int64_t chunk = (e1 - e0 + psplit - 1) / psplit;
     const int64_t l0 = e0 + blockIdx.y * chunk, l1 = min(e1, l0 + chunk);
-    L acc[3] = {0, 0, 0};
-    const L eta_c = VMODE == PG_LAM_R ? eta[c] : L(0);
+    double acc[3] = {0, 0, 0};
     // a thread's entries e0, e0 + 256, ... taken PGU at a time: the loads of PGU entries (row
     // index, then the gathered value) in flight together, the products added in ascending e
     constexpr int PGU = 8;
     for (int64_t e0 = l0 + threadIdx.x; e0 < l1; e0 += PGU * (int64_t)blockDim.x) {
         int64_t rr[PGU];
-        L xv[PGU];
+        double xv[PGU];
 #pragma unroll
         for (int m = 0; m < PGU; ++m) {
             const int64_t e = e0 + (int64_t)m * blockDim.x;
@@ -816,11 +515,10 @@ __global__ void __launch_bounds__(256) k_proj_g(const int64_t *range, const int3
 #pragma unroll
         for (int m = 0; m < PGU; ++m) {
             const int64_t e = e0 + (int64_t)m * blockDim.x;
-            L x = 0;
+            double x = 0;
             if (e < l1) {
                 if (VMODE == PG_U) x = v[e * R + c];
-                else if (VMODE == PG_LAM) x = v[rr[m] * R + c];
-                else x = r_next(v[rr[m] * R + c], q[rr[m] * R + c], eta_c);
+                else x = v[rr[m] * R + c];
             }
             xv[m] = x;
         }
@@ -839,39 +537,11 @@ __global__ void __launch_bounds__(256) k_proj_g(const int64_t *range, const int3
         for (int q = 0; q < 3; ++q) red[warp][q] = acc[q];
     __syncthreads();
     if (threadIdx.x < nq) {
-        L x = 0;
+        double x = 0;
         for (int ww = 0; ww < 8; ++ww) x += red[ww][threadIdx.x];
         gpart[((int64_t)(co_off + threadIdx.x) * psplit + blockIdx.y) * R + c] = (double)x;
     }
     if (!fused) return;
-    if constexpr (std::is_same<L, float>::value) {
-        if (fused == 2) {
-            if (!arrive_last_col(colcnt, c)) return;
-            float *gc = reinterpret_cast<float *>(gs_dyn);       // n_co entries of G^T v, column c
-            for (int j = threadIdx.x; j < nco; j += blockDim.x) {
-                double g = 0;
-                for (int s = 0; s < psplit; ++s) g += __ldcg(gpart + ((int64_t)j * psplit + s) * R + c);
-                gc[j] = (float)g;
-            }
-            __syncthreads();
-            for (int i = threadIdx.x; i < nco; i += blockDim.x) {
-                // j ascending; the loads of 16 consecutive j in flight together
-                float a = 0.0f;
-                int j = 0;
-                for (; j + 16 <= nco; j += 16) {
-                    float gv[16];
-#pragma unroll
-                    for (int m = 0; m < 16; ++m) gv[m] = __ldg(GtGinv32 + (int64_t)(j + m) * nco + i);
-#pragma unroll
-                    for (int m = 0; m < 16; ++m) a = __fmaf_rn(gv[m], gc[j + m], a);
-                }
-                for (; j < nco; ++j) a = __fmaf_rn(__ldg(GtGinv32 + (int64_t)j * nco + i), gc[j], a);
-                alpha[(int64_t)i * R + c] = a;
-            }
-            if (threadIdx.x == 0) colcnt[c] = 0u;
-            return;
-        }
-    }
     if (!arrive_last(counter)) return;
     double *gs = gsum ? gsum : gs_dyn;
     for (int t = threadIdx.x; t < nco * R; t += blockDim.x) {
@@ -885,7 +555,7 @@ __global__ void __launch_bounds__(256) k_proj_g(const int64_t *range, const int3
         const int i = t / R, cc = t % R;
         double a = 0;
         for (int j = 0; j < nco; ++j) a += GtGinv[(int64_t)i * nco + j] * gs[(int64_t)j * R + cc];
-        alpha[t] = (L)a;
+        alpha[t] = (double)a;
     }
     if (threadIdx.x == 0) *counter = 0u;
 }
@@ -910,6 +580,7 @@ __global__ void __launch_bounds__(256) k_coarse_solve(const double *gpart, int p
 }
 
 #include "lambda_cluster.cuh"
+#include "lambda_rows.cuh"
 
 // refinement update u += du with corr = max |du| / max |u| per column: grid (row blocks,
 // right-hand sides), per-block maxima, the last block to arrive writes corr (maxima do not
@@ -1437,18 +1108,6 @@ struct Runner {
         if constexpr (std::is_same<L, float>::value) return d32.as<float>();
         else return d64.as<double>();
     }
-    template <typename L> const L *eta_ptr() const {
-        if constexpr (std::is_same<L, float>::value) return S.eta_f;
-        else return S.eta;
-    }
-    template <typename L> const L *beta_ptr() const {
-        if constexpr (std::is_same<L, float>::value) return S.beta_f;
-        else return S.beta;
-    }
-    template <typename L> const L *xscale_ptr() const {
-        if constexpr (std::is_same<L, float>::value) return S.xscale_f;
-        else return ws.xscale.as<double>();
-    }
     // the PCG vectors of the iterations (r, w, z, y, p, q, lambda) in L
     template <typename L> struct LamVecs { L *r, *w, *z, *y, *pv, *q, *lam; };
     template <typename L> LamVecs<L> lam_vecs() {
@@ -1462,37 +1121,43 @@ struct Runner {
         }
     }
 
-    // alpha = (G^T G)^-1 G^T v: v on U (PG_U, FP64), on Lambda (PG_LAM) or r_new = v - eta q
-    // (PG_LAM_R); alpha in L
-    template <typename L> void coarse_alpha(const L *v, int vmode, const L *q = nullptr) {
+    // alpha = (G^T G)^-1 G^T v in FP64: v on U (PG_U) or on Lambda (PG_LAM)
+    void coarse_alpha(const double *v, int vmode) {
+        const bool fused = p->n_co <= kCoarseFusedMax;
+        const int psplit = fused ? PSPLIT : 1;
+        const size_t gs_bytes = sizeof(double) * (size_t)p->n_co * R;
+        const bool in_smem = fused && gs_bytes <= 32768;
+        double *alpha = ws.alpha.as<double>();
+        auto go = [&](auto kern, const double *w) {
+            kern<<<dim3(p->n_floating, psplit, R), 256, in_smem ? gs_bytes : 0, st>>>(
+                p->d_gt_range.as<int64_t>(), p->d_gt_co.as<int32_t>(), p->d_gt_rows.as<int64_t>(), w, v,
+                ws.gco.as<double>(), in_smem ? nullptr : ws.gsum.as<double>(), p->d_GtGinv.as<double>(), p->n_co, alpha, R,
+                S.counter, psplit, fused ? 1 : 0);
+        };
+        if (vmode == PG_U) go(k_proj_g<PG_U>, p->d_Z.as<double>());
+        else go(k_proj_g<PG_LAM>, p->d_gt_w.as<double>());
+        note_launch();
+        if (!fused) coarse_solve<double>(psplit, alpha);
+    }
+    template <typename L> void coarse_solve(int psplit, L *alpha) {
+        k_coarse_solve<L><<<dim3((p->n_co + 7) / 8, R), 256, 0, st>>>(ws.gco.as<double>(), psplit,
+                                                                     p->d_GtGinv.as<double>(), p->n_co, alpha, R);
+        note_launch();
+    }
+
+    // the same inside the iterations, in L: v = z or (RNEW) r_new = r - eta q
+    template <int RNEW, typename L, int V> void coarse_iter(const LamArgs<L> &a) {
         const bool fused = p->n_co <= kCoarseFusedMax;
         const bool colfused = std::is_same<L, float>::value && !fused && p->n_co <= kCoarseColMax;
         const int psplit = fused ? PSPLIT : 1;
         const size_t gs_bytes = sizeof(double) * (size_t)p->n_co * R;
         const bool in_smem = fused && gs_bytes <= 32768;
-        const size_t smem = in_smem ? gs_bytes : (colfused ? sizeof(float) * (size_t)p->n_co : 0);
+        const size_t smem = in_smem ? gs_bytes : (colfused ? sizeof(float) * (size_t)p->n_co * V : 0);
         L *alpha = ws.alpha.as<L>();
-        auto go = [&](auto kern, const L *w) {
-            kern<<<dim3(p->n_floating, psplit, R), 256, smem, st>>>(
-                p->d_gt_range.as<int64_t>(), p->d_gt_co.as<int32_t>(), p->d_gt_rows.as<int64_t>(), w, v, q,
-                eta_ptr<L>(), ws.gco.as<double>(), in_smem ? nullptr : ws.gsum.as<double>(), p->d_GtGinv.as<double>(),
-                p->n_co, alpha, R, S.counter, psplit, fused ? 1 : (colfused ? 2 : 0), p->d_GtGinv32.as<float>(),
-                S.colcnt);
-        };
-        if (vmode == PG_U) {
-            if constexpr (std::is_same<L, double>::value) go(k_proj_g<PG_U, double>, p->d_Z.as<double>());
-            else fail(NLFETI_E_INVALID, "the U-space coarse gather runs in FP64");
-        } else if (vmode == PG_LAM) {
-            go(k_proj_g<PG_LAM, L>, wt<L>(p->d_gt_w, p->d_gt_w32));
-        } else {
-            go(k_proj_g<PG_LAM_R, L>, wt<L>(p->d_gt_w, p->d_gt_w32));
-        }
+        k_proj_v<RNEW, L, V><<<dim3(p->n_floating, psplit, R / V), 256, smem, st>>>(
+            a, ws.gco.as<double>(), in_smem ? nullptr : ws.gsum.as<double>(), alpha, psplit, fused ? 1 : (colfused ? 2 : 0));
         note_launch();
-        if (!fused && !colfused) {
-            k_coarse_solve<L><<<dim3((p->n_co + 7) / 8, R), 256, 0, st>>>(ws.gco.as<double>(), psplit,
-                                                                         p->d_GtGinv.as<double>(), p->n_co, alpha, R);
-            note_launch();
-        }
+        if (!fused && !colfused) coarse_solve<L>(psplit, alpha);
     }
 
     // out = P v (out may alias v)
@@ -1505,17 +1170,6 @@ struct Runner {
         coarse_alpha(v, PG_LAM);
         k_apply_galpha<<<grid_for(nl * R), 256, 0, st>>>(p->d_Gcol.as<int32_t>(), p->d_Gval.as<double>(), p->gw,
                                                          ws.alpha.as<double>(), v, -1.0, out, nl, R);
-        note_launch();
-    }
-
-    // out = P v with the PCG dot product of MODE fused in (CHECK: (out, out); BETA: (out, other))
-    template <int MODE, typename L> void project_dot(const L *v, const L *other, L *out, double tol = 0,
-                                                     int max_it = 0) {
-        const int64_t nl = p->n_lambda;
-        if (p->n_co > 0) coarse_alpha<L>(v, PG_LAM);
-        k_project_dot<MODE, L><<<tile_blocks(nl), TILE_THREADS, 0, st>>>(
-            p->d_Gcol.as<int32_t>(), wt<L>(p->d_Gval, p->d_Gval32), p->gw, p->n_co > 0 ? ws.alpha.as<L>() : nullptr, v,
-            other, out, nl, R, ws.partial.as<double>(), S, tol, max_it);
         note_launch();
     }
 
@@ -1816,30 +1470,15 @@ struct Runner {
                pool.St.p && ws.xhmaps.p;
     }
 
-    // out = M^-1 v (the scaled Dirichlet preconditioner), v and out in L
-    template <typename T, typename L = double>
-    void applyMinv(const OpPool<T> &pool, const L *v, L *out, bool precond = false) {
+    // out = M^-1 v (the scaled Dirichlet preconditioner)
+    template <typename T> void applyMinv(const OpPool<T> &pool, const double *v, double *out) {
         const int64_t nl = p->n_lambda, nu = p->n_u;
         T *x = apply_input<T>(ws);
-        float *const saved_out = yout_f;
-        yout_f = std::is_same<L, float>::value ? ws.yU.as<float>() : nullptr;   // y_U in L
-        if (use_mma(pool, precond)) {
-            if (nu > 0) {
-                k_gather_apply_f16<L><<<grid_for(nu * R), 256, 0, st>>>(
-                    p->d_BDt_ptr.as<int64_t>(), p->d_BDt_row.as<int64_t>(), wt<L>(p->d_BDt_val, p->d_BDt_val32), v,
-                    xscale_ptr<L>(), ws.xU.as<__half>(), sd, p->d_u2sub.as<int32_t>(), nu, R, gate);
-                note_launch();
-                symv_mma(pool, ws.yU.as<double>());
-            }
-        } else {
-            if (nu > 0)
-                gather_x<T, L>(p->d_BDt_ptr.as<int64_t>(), p->d_BDt_row.as<int64_t>(),
-                               wt<L>(p->d_BDt_val, p->d_BDt_val32), v, x);
-            symv<T>(pool, 0, x, ws.yU.as<double>(), precond);
-        }
-        yout_f = saved_out;
-        k_gather_bd<L><<<grid_for(nl * R), 256, 0, st>>>(p->d_BD_ptr.as<int64_t>(), p->d_BD_col.as<int64_t>(),
-                                                         wt<L>(p->d_BD_val, p->d_BD_val32), ws.yU.as<L>(), out, nl, R);
+        if (nu > 0)
+            gather_x<T, double>(p->d_BDt_ptr.as<int64_t>(), p->d_BDt_row.as<int64_t>(), p->d_BDt_val.as<double>(), v, x);
+        symv<T>(pool, 0, x, ws.yU.as<double>());
+        k_gather_bd<double><<<grid_for(nl * R), 256, 0, st>>>(p->d_BD_ptr.as<int64_t>(), p->d_BD_col.as<int64_t>(),
+                                                              p->d_BD_val.as<double>(), ws.yU.as<double>(), out, nl, R);
         note_launch();
     }
 
@@ -1954,41 +1593,47 @@ struct Runner {
     // FP64 in both.
     template <typename T> void iteration(const OpPool<T> &pool, double tol, int max_it) {
         if (p->lam_ok) return iteration_clusters<T>(pool, tol, max_it);
+        if constexpr (std::is_same<T, float>::value) {
+            if (R % 4 == 0) return iteration_rows<T, 4>(pool, tol, max_it);
+            if (R % 2 == 0) return iteration_rows<T, 2>(pool, tol, max_it);
+        }
+        iteration_rows<T, 1>(pool, tol, max_it);
+    }
+
+    template <typename T, int V> void iteration_rows(const OpPool<T> &pool, double tol, int max_it) {
         using L = T;
         const int64_t nl = p->n_lambda, nu = p->n_u;
+        LamArgs<L> a = lam_args<L>(tol, max_it);
         const LamVecs<L> v = lam_vecs<L>();
-        L *yU = ws.yU.as<L>();          // the applies' output, in L
-        T *x = apply_input<T>(ws);
+        a.r = v.r; a.w = v.w; a.z = v.z; a.y = v.y; a.pv = v.pv; a.q = v.q; a.lam = v.lam;
+        const bool mma = use_mma(pool, true);
+        a.x16 = mma ? ws.xU.as<__half>() : nullptr;
         const L *alpha = p->n_co > 0 ? ws.alpha.as<L>() : nullptr;
+        auto *partial = ws.partial.as<typename PartialOf<L>::type>();
         // p, lambda, r updated; w = P r, ||w||, stop test
-        if (p->n_co > 0) coarse_alpha<L>(v.r, PG_LAM_R, v.q);
-        auto check = [&](auto kern) {
-            kern<<<tile_blocks(nl), TILE_THREADS, 0, st>>>(p->d_Gcol.as<int32_t>(), wt<L>(p->d_Gval, p->d_Gval32), p->gw,
-                                                          alpha, v.y, v.pv, v.lam, v.r, v.q, v.w, nl, R,
-                                                          ws.partial.as<double>(), S, tol, max_it, cond, max_it + 1);
-        };
-        if (use_cond) check(k_check_update<1, L>);
-        else check(k_check_update<0, L>);
+        if (p->n_co > 0) coarse_iter<1, L, V>(a);
+        if (use_cond) k_check_update<1, L, V><<<tile_blocks(nl), TILE_THREADS, 0, st>>>(a, alpha, partial);
+        else k_check_update<0, L, V><<<tile_blocks(nl), TILE_THREADS, 0, st>>>(a, alpha, partial);
         note_launch();
         gate = S.n_active;
-        applyMinv<T, L>(pool, v.w, v.z, true);                   // z = M^-1 w
-        project_dot<FIN_BETA, L>(v.z, v.w, v.y);                 // y = P z, (y, w), beta
-        // q = F p_new, (p_new, q), eta
-        if (R <= GX_MAXR)
-            k_gather_apply_p_t<T, L><<<(unsigned)((nu + GX_U - 1) / GX_U), 256, sizeof(double) * GX_U * R, st>>>(
-                p->d_Bt_ptr.as<int64_t>(), p->d_Bt_row.as<int64_t>(), v.pv, v.y, beta_ptr<L>(), S.active, x, sd,
-                p->d_u2sub.as<int32_t>(), nu, R, gate);
-        else
-            k_gather_apply_p<T, L><<<grid_for(nu * R), 256, 0, st>>>(p->d_Bt_ptr.as<int64_t>(),
-                                                                     p->d_Bt_row.as<int64_t>(), v.pv, v.y,
-                                                                     beta_ptr<L>(), S.active, x, sd,
-                                                                     p->d_u2sub.as<int32_t>(), nu, R, gate);
-        note_launch();
         yout_f = std::is_same<L, float>::value ? ws.yU.as<float>() : nullptr;
-        symv<T>(pool, 1, x, ws.yU.as<double>());
+        // z = M^-1 w
+        k_gather_w_v<L, V><<<grid_for(nu * (R / V)), 256, 0, st>>>(a, p->d_l_u2c.as<int4>(), gate);
+        note_launch();
+        if (mma) symv_mma(pool, ws.yU.as<double>());
+        else symv<T>(pool, 0, apply_input<T>(ws), ws.yU.as<double>(), true);
+        k_gather_bd_v<L, V><<<grid_for(nl * (R / V)), 256, 0, st>>>(a);
+        note_launch();
+        // y = P z, (y, w), beta
+        if (p->n_co > 0) coarse_iter<0, L, V>(a);
+        k_project_dot<L, V><<<tile_blocks(nl), TILE_THREADS, 0, st>>>(a, alpha, partial);
+        note_launch();
+        // q = F p_new, (p_new, q), eta
+        k_gather_p_v<L, V><<<grid_for(nu * (R / V)), 256, 0, st>>>(a, gate);
+        note_launch();
+        symv<T>(pool, 1, apply_input<T>(ws), ws.yU.as<double>());
         yout_f = nullptr;
-        k_gather_b_eta<L><<<tile_blocks(nl), TILE_THREADS, 0, st>>>(p->d_Bp.as<int64_t>(), p->d_Bm.as<int64_t>(), yU,
-                                                                  v.pv, v.y, v.q, nl, R, ws.partial.as<double>(), S);
+        k_gather_b_eta<L, V><<<tile_blocks(nl), TILE_THREADS, 0, st>>>(a, partial);
         note_launch();
         gate = nullptr;
     }

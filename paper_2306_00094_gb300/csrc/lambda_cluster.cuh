@@ -6,7 +6,7 @@
 //   k_lam_a (after S^+):  q = B y_U, (p, q), eta;  G^T r_new, alpha;  p, lambda, r, w = P r, (w, w),
 //                         stop test;  x = B_D^T w;
 //   k_lam_b (after S):    z = B_D y_U;  G^T z, alpha;  y = P z, (y, w), beta;  x = B^T p_new.
-// As one kernel per step they are latency-bound: a launch with a fused reduction takes 7-10 us even
+// As one kernel per step (lambda_rows.cuh) they are latency-bound: a launch with a fused reduction takes 7-10 us even
 // on a few hundred rows (start-up, fence, arrival atomic, the last block's finish), where the data
 // (a few MB, resident in L2) would take one or two.  The right-hand sides of a PCG are independent
 // of one another, so a cluster of LC CTAs (16 SMs of one GPC) owns CW of them for the whole kernel,
@@ -378,7 +378,7 @@ __device__ __forceinline__ void lam_store_x(const LamArgs<L> &a, int u, int c0, 
     if constexpr (std::is_same<L, float>::value) {
         const int R2 = (a.R + 1) / 2 * 2;
         L *p = a.x + (size_t)t.x * R2 + (size_t)(c0 >> 1) * t.y + t.z;
-        if constexpr (CW == 1) p[0] = v[0];
+        if constexpr (CW == 1) p[c0 & 1] = v[0];
         else
 #pragma unroll
             for (int c = 0; c < CW; c += 2)

@@ -1104,7 +1104,7 @@ void setup_lambda(nlfeti_problem *p) {
     int zmax = 0;                    // most copies of a node: entries of a B_D row (one less per B_D^T row)
     for (int32_t z : p->dec.node_zeta) zmax = std::max(zmax, (int)z);
     p->lam_ok = lambda_clusters_ok(p, zmax);
-    if (!p->lam_ok) return;
+    if (nl == 0) return;
     p->lam_bd_w = zmax;
     p->lam_bdt_w = zmax - 1;
     auto I = [&](DevMem &m, int64_t n) { m.alloc(c, sizeof(int32_t) * std::max<int64_t>(1, n)); return m.as<int32_t>(); };
