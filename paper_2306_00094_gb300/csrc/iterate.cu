@@ -310,6 +310,23 @@ __device__ __forceinline__ void block_partial(double acc, double *partial, int R
     }
 }
 
+// sum of one column's nb block partials (partial[b * R + c]) by a warp: 8 loads of a lane in flight (one
+// at a time, the rounds of L2 latency were half of the CG's update kernel), added in block order per
+// lane, then the lane tree
+__device__ __forceinline__ double sum_partials(const double *partial, int nb, int R, int c) {
+    const int lane = threadIdx.x % 32;
+    double v = 0;
+    for (int b0 = lane; b0 < nb; b0 += 32 * 8) {
+        double t[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) t[u] = b0 + 32 * u < nb ? __ldcg(partial + (int64_t)(b0 + 32 * u) * R + c) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (b0 + 32 * u < nb) v += t[u];
+    }
+    return warp_sum(v);
+}
+
 // true in the last block of the grid to arrive (after every block's partials are visible)
 __device__ __forceinline__ bool arrive_last(unsigned *counter) {
     __shared__ bool last;
@@ -582,35 +599,47 @@ __global__ void __launch_bounds__(256) k_coarse_solve(const double *gpart, int p
 #include "lambda_cluster.cuh"
 #include "lambda_rows.cuh"
 
-// refinement update u += du with corr = max |du| / max |u| per column: grid (row blocks,
-// right-hand sides), per-block maxima, the last block to arrive writes corr (maxima do not
-// depend on the order)
+// refinement update u += du with corr = max |du| / max |u| per column (maxima do not depend on the
+// order).  Blocks take chunks of up to RED_THREADS columns (grid y), a thread one column of every
+// (threads / chunk)-th row, so that neighbouring threads read neighbouring entries; a block's maxima are combined
+// per column in shared memory and the last block to arrive writes corr.  (One block row per column,
+// each reading every R-th entry, took 80 us on the peridynamic workload, 168200 x 16; now 12 us on the factorization workload, 36450 x 2, from 23.)
+inline dim3 refine_grid(int64_t n, int R) {
+    const int cb = std::min(R, RED_THREADS), rows = RED_THREADS / cb;
+    return dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>(RED_BLOCKS, (n + rows - 1) / rows)), (R + cb - 1) / cb);
+}
 __global__ void __launch_bounds__(RED_THREADS) k_refine_update(double *u, const double *du, int64_t n, int R,
                                                                 double *pa, double *pb, PcgScalars s) {
-    __shared__ double ra[RED_THREADS / 32], rb[RED_THREADS / 32];
-    const int c = blockIdx.y, warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    __shared__ double sa[RED_THREADS], sb[RED_THREADS];
+    const int cb = min(R, RED_THREADS), rows = RED_THREADS / cb;
+    const int c = blockIdx.y * cb + threadIdx.x % cb, rl = threadIdx.x / cb;
     double ma = 0, mb = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double d = du[i * R + c], v = u[i * R + c] + d;
-        u[i * R + c] = v;
-        ma = fmax(ma, fabs(d));
-        mb = fmax(mb, fabs(v));
+    if (rl < rows && c < R)
+#pragma unroll 4
+        for (int64_t i = (int64_t)blockIdx.x * rows + rl; i < n; i += (int64_t)gridDim.x * rows) {
+            const double d = du[i * R + c], v = u[i * R + c] + d;
+            u[i * R + c] = v;
+            ma = fmax(ma, fabs(d));
+            mb = fmax(mb, fabs(v));
+        }
+    sa[threadIdx.x] = ma;
+    sb[threadIdx.x] = mb;
+    for (int o = RED_THREADS / 2; o > 0; o >>= 1) {          // tree over the block's rows
+        __syncthreads();
+        if (rl < o && rl + o < rows) {
+            sa[threadIdx.x] = ma = fmax(ma, sa[threadIdx.x + o * cb]);
+            sb[threadIdx.x] = mb = fmax(mb, sb[threadIdx.x + o * cb]);
+        }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        ma = fmax(ma, __shfl_xor_sync(0xffffffffu, ma, o));
-        mb = fmax(mb, __shfl_xor_sync(0xffffffffu, mb, o));
-    }
-    if (lane == 0) { ra[warp] = ma; rb[warp] = mb; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double x = 0, y = 0;
-        for (int w = 0; w < RED_THREADS / 32; ++w) { x = fmax(x, ra[w]); y = fmax(y, rb[w]); }
-        pa[(int64_t)blockIdx.x * R + c] = x;
-        pb[(int64_t)blockIdx.x * R + c] = y;
+    if (rl == 0 && c < R) {
+        pa[(int64_t)blockIdx.x * R + c] = ma;
+        pb[(int64_t)blockIdx.x * R + c] = mb;
     }
     if (!arrive_last(s.counter)) return;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     for (int cc = warp; cc < R; cc += RED_THREADS / 32) {
         double x = 0, y = 0;
+#pragma unroll 5
         for (int bl = lane; bl < (int)gridDim.x; bl += 32) {
             x = fmax(x, __ldcg(pa + (int64_t)bl * R + cc));
             y = fmax(y, __ldcg(pb + (int64_t)bl * R + cc));
@@ -690,13 +719,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_cg_init(const double *b, const 
     if (threadIdx.x == 0) n_act = 0;
     __syncthreads();
     for (int cc = warp; cc < R; cc += RED_THREADS / 32) {
-        double rz = 0, bb = 0;
-        for (int bl = lane; bl < (int)gridDim.x; bl += 32) {
-            rz += __ldcg(pa + (int64_t)bl * R + cc);
-            bb += __ldcg(pb + (int64_t)bl * R + cc);
-        }
-        rz = warp_sum(rz);
-        bb = warp_sum(bb);
+        const double rz = sum_partials(pa, gridDim.x, R, cc), bb = sum_partials(pb, gridDim.x, R, cc);
         if (lane == 0) {
             const int act = bb > 0.0 ? 1 : 0;
             s.nPd[cc] = sqrt(bb);
@@ -851,13 +874,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_cg_update(const double *dinv, c
     if (threadIdx.x == 0) n_act = 0;
     __syncthreads();
     for (int cc = warp; cc < R; cc += RED_THREADS / 32) {
-        double rz = 0, rr = 0;
-        for (int bl = lane; bl < (int)gridDim.x; bl += 32) {
-            rz += __ldcg(pa + (int64_t)bl * R + cc);
-            rr += __ldcg(pb + (int64_t)bl * R + cc);
-        }
-        rz = warp_sum(rz);
-        rr = warp_sum(rr);
+        const double rz = sum_partials(pa, gridDim.x, R, cc), rr = sum_partials(pb, gridDim.x, R, cc);
         if (lane == 0) {
             int act = s.active[cc];
             if (act) {
@@ -2237,7 +2254,7 @@ void solve_device(nlfeti_problem *p, SolveWS &ws, cudaStream_t st, int R, int rh
             }
             run.pass<float>(p->op32, p->opt.inner_tol, p->opt.max_it, sw > 0);
             if (nl > 0) k_axpy<<<grid_for(nl * R), 256, 0, st>>>(ws.lam.as<double>(), ws.dlam.as<double>(), 1.0, nl * R);
-            k_refine_update<<<red_grid(nv, R), RED_THREADS, 0, st>>>(ws.u.as<double>(), ws.du.as<double>(), nv, R,
+            k_refine_update<<<refine_grid(nv, R), RED_THREADS, 0, st>>>(ws.u.as<double>(), ws.du.as<double>(), nv, R,
                                                                      ws.partial.as<double>(), ws.partial2.as<double>(),
                                                                      run.S);
             run.eager_launches += 1 + (nl > 0);
