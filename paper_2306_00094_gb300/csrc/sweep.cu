@@ -14,12 +14,11 @@
 //
 // Pivot blocks are NB = 64 wide; a step is three launches over all subdomains: invert
 // the pivot block (one CTA per subdomain), form the pivot panels, update all tiles.  FP64: on the
-// tensor cores by exact digit products, block upper triangle only (sweep_dg.cuh).  FP32: 64x64 CTA
-// tiles, 4x4 register blocking, or per the factor_tc option 128x128 tiles on the tensor cores,
-// split-TF32, in sweep_tc.cuh: by default in the Omega sweep of A^k, the sweep of the pinned S_k
-// staying on the FP32 pipes.  A non-positive pivot sets the device status word (NLFETI_E_NOT_SPD)
+// tensor cores by exact digit products, block upper triangle only (sweep_dg.cuh).  FP32: likewise
+// (sweep_d4.cuh), or with factor_tc = 0 64x64 CTA tiles, 4x4 register blocking, on the FP32 pipes.  A non-positive pivot sets the device status word (NLFETI_E_NOT_SPD)
 // instead of trapping.
 #include <algorithm>
+#include <numeric>
 #include <type_traits>
 #include <cmath>
 #include <cstring>
@@ -72,28 +71,6 @@ __device__ bool sweep_block_shared(T *S, int n, int ld, T *rowp) {
     }
     __syncthreads();
     return ok;
-}
-
-template <typename T> __global__ void k_pivot(SweepArgs<T> a) {
-    const int k = blockIdx.x;
-    const int pend = a.pend[k];
-    if (a.j0 >= pend) return;
-    const int b = min(NB, pend - a.j0);
-    const int ld = a.mld[k];
-    T *M = a.M + a.moff[k];
-    __shared__ T S[NB * NB];
-    __shared__ T rowp[NB];
-    for (int t = threadIdx.x; t < b * b; t += blockDim.x) {
-        int i = t / b, l = t % b;
-        S[i * NB + l] = M[(int64_t)(a.j0 + i) * ld + a.j0 + l];
-    }
-    bool ok = sweep_block_shared(S, b, NB, rowp);
-    if (!ok && threadIdx.x == 0) atomicMax(a.flag, 1);
-    T *D = a.dinv + (int64_t)k * NB * NB;
-    for (int t = threadIdx.x; t < b * b; t += blockDim.x) {
-        int i = t / b, l = t % b;
-        D[i * NB + l] = -S[i * NB + l];       // D^-1
-    }
 }
 
 // panels: old_i = M_iJ, pan_i = M_iJ D^-1 for every row i
@@ -184,6 +161,7 @@ template <typename T> __global__ void __launch_bounds__(256) k_update(SweepArgs<
 
 #include "sweep_tc.cuh"
 #include "sweep_dg.cuh"
+#include "sweep_d4.cuh"
 
 // copy A^k (FP64, ld = nk) into the swept-matrix pool (type T, ld = ldM, zero padding)
 template <typename T> __global__ void k_load_matrix(const double *A, T *Mpool, const SubdomainDesc *sd) {
@@ -526,7 +504,106 @@ void run_sweeps_dg(nlfeti_problem *p, double *pool, const std::vector<int64_t> &
         k_update_dg<<<dim3(nt, chunks, K), DG_THREADS, DG_SMEM_UPD, c->stream>>>(a);
     }
     const unsigned mt = (unsigned)((maxn + 31) / 32);
-    k_mirror_up<<<dim3(mt, mt, K), 256, 0, c->stream>>>(pool, a.moff, a.mdim, a.mld);
+    k_mirror_up<double><<<dim3(mt, mt, K), 256, 0, c->stream>>>(pool, a.moff, a.mdim, a.mld);
+    NLF_CUDA(cudaGetLastError());
+    NLF_CUDA(cudaStreamSynchronize(c->stream));
+}
+
+// the FP32 sweeps on the tensor cores (sweep_d4.cuh)
+void run_sweeps_d4(nlfeti_problem *p, float *pool, const std::vector<int64_t> &moff, const std::vector<int32_t> &mdim,
+                   const std::vector<int32_t> &mld, const std::vector<int32_t> &pend, DevMem &scratch) {
+    nlfeti_ctx *c = p->ctx;
+    const int K = p->K;
+    std::vector<int64_t> soff(K);
+    int64_t rows = 0;
+    int maxn = 0, maxp = 0;
+    for (int k = 0; k < K; ++k) {
+        soff[k] = rows;
+        rows += (mdim[k] + DG_TILE - 1) / DG_TILE * DG_TILE;
+        maxn = std::max(maxn, mdim[k]);
+        maxp = std::max(maxp, pend[k]);
+    }
+    if (maxp == 0) return;
+    const size_t dbytes = (size_t)(rows / DG_TILE) * D4 * DG_TBYTES;
+    const size_t need = 2 * dbytes + sizeof(float) * (2 * (size_t)rows + (size_t)K * NB * NB) + sizeof(int) * (size_t)K * NB;
+    if (scratch.bytes < need) scratch.alloc(c, need);
+    DevMem d_moff, d_mdim, d_mld, d_pend, d_soff;
+    upload(c, d_moff, moff);
+    upload(c, d_mdim, mdim);
+    upload(c, d_mld, mld);
+    upload(c, d_pend, pend);
+    upload(c, d_soff, soff);
+    Digit4Args a;
+    a.M = pool;
+    a.pan_d = scratch.as<unsigned char>();
+    a.old_d = a.pan_d + dbytes;
+    a.pan = a.old = nullptr;
+    a.dinv = reinterpret_cast<float *>(a.old_d + dbytes);
+    a.pan_s = a.dinv + (size_t)K * NB * NB;
+    a.old_s = a.pan_s + rows;
+    a.piv_c = reinterpret_cast<int *>(a.old_s + rows);
+    a.sd = p->d_sd.as<SubdomainDesc>();
+    a.moff = d_moff.as<int64_t>();
+    a.mdim = d_mdim.as<int32_t>();
+    a.mld = d_mld.as<int32_t>();
+    a.pend = d_pend.as<int32_t>();
+    a.scr_off = d_soff.as<int64_t>();
+    a.flag = p->d_flag.as<int>();
+    NLF_CUDA(cudaFuncSetAttribute(k_panel_d4, cudaFuncAttributeMaxDynamicSharedMemorySize, D4_SMEM_PAN));
+    NLF_CUDA(cudaFuncSetAttribute(k_update_d4, cudaFuncAttributeMaxDynamicSharedMemorySize, D4_SMEM_UPD));
+    const unsigned nt = (unsigned)((maxn + DG_TILE - 1) / DG_TILE);
+    // The update's work: the blocks of the columns of the subdomains that have pivots left, split evenly
+    // over one CTA per SM (at least a block each), rebuilt when a subdomain is done
+    const int sms = device_sms();
+    std::vector<int4> segs;
+    std::vector<int32_t> seg_ptr;
+    struct Phase { int j0; size_t seg, ptr; unsigned ctas; };
+    std::vector<Phase> phases;
+    std::vector<int> ends(pend.begin(), pend.end());
+    std::sort(ends.begin(), ends.end());
+    for (int j0 = 0; j0 < maxp; j0 += NB) {
+        // subdomains leave between the step before and this one?
+        if (j0 > 0 && std::upper_bound(ends.begin(), ends.end(), j0) == std::upper_bound(ends.begin(), ends.end(), j0 - NB))
+            continue;
+        int64_t blocks = 0, done = 0;
+        for (int k = 0; k < K; ++k) {
+            const int64_t t = (mdim[k] + DG_TILE - 1) / DG_TILE;
+            if (pend[k] > j0) blocks += t * (t + 1) / 2;
+        }
+        const int64_t ctas = std::min<int64_t>(sms, blocks);
+        phases.push_back({j0, segs.size(), seg_ptr.size(), (unsigned)ctas});
+        const size_t base = segs.size();
+        int64_t g = 0;
+        seg_ptr.push_back(0);
+        for (int k = 0; k < K; ++k)
+            for (int t = 0; pend[k] > j0 && t < (mdim[k] + DG_TILE - 1) / DG_TILE; ++t)
+                for (int q = 0; q <= t;) {
+                    const int64_t end = (g + 1) * blocks / ctas;          // of CTA g
+                    const int e = (int)std::min<int64_t>(t + 1, q + end - done);
+                    segs.push_back(make_int4(k, t, q, e));
+                    done += e - q;
+                    q = e;
+                    if (done == end) {
+                        seg_ptr.push_back((int32_t)(segs.size() - base));
+                        ++g;
+                    }
+                }
+    }
+    DevMem d_segs, d_seg_ptr;
+    upload(c, d_segs, segs);
+    upload(c, d_seg_ptr, seg_ptr);
+    size_t phase = 0;
+    for (int j0 = 0; j0 < maxp; j0 += NB) {
+        a.j0 = j0;
+        k_pivot_f32<<<K, PIV_THREADS, 0, c->stream>>>(a, a.piv_c);
+        k_panel_d4<<<dim3(nt, K), D4_PAN_THREADS, D4_SMEM_PAN, c->stream>>>(a);
+        if (phase + 1 < phases.size() && phases[phase + 1].j0 == j0) ++phase;
+        a.segs = d_segs.as<int4>() + phases[phase].seg;
+        a.seg_ptr = d_seg_ptr.as<int32_t>() + phases[phase].ptr;
+        k_update_d4<<<phases[phase].ctas, D4_THREADS, D4_SMEM_UPD, c->stream>>>(a);
+    }
+    const unsigned mt = (unsigned)((maxn + 31) / 32);
+    k_mirror_up<float><<<dim3(mt, mt, K), 256, 0, c->stream>>>(pool, a.moff, a.mdim, a.mld);
     NLF_CUDA(cudaGetLastError());
     NLF_CUDA(cudaStreamSynchronize(c->stream));
 }
@@ -536,6 +613,7 @@ template <typename T> void run_sweeps(nlfeti_problem *p, T *pool, const std::vec
                                       const std::vector<int32_t> &pend, DevMem &scratch, bool allow_tc) {
     if constexpr (std::is_same<T, double>::value) return run_sweeps_dg(p, pool, moff, mdim, mld, pend, scratch);
     else {
+    if (allow_tc) return run_sweeps_d4(p, pool, moff, mdim, mld, pend, scratch);
     nlfeti_ctx *c = p->ctx;
     const int K = p->K;
     std::vector<int64_t> soff(K);
@@ -571,20 +649,10 @@ template <typename T> void run_sweeps(nlfeti_problem *p, T *pool, const std::vec
     const int nt = (maxn + TILE - 1) / TILE;
     const size_t smu = sizeof(T) * 2 * NB * TILE;
     NLF_CUDA(cudaFuncSetAttribute(k_update<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smu));
-    // FP32 operators with factor_tc: the rank-64 updates on the tensor cores (split-TF32)
-    const bool tc = std::is_same<T, float>::value && allow_tc;
-    const int ntc = (maxn + TC_TILE - 1) / TC_TILE;
-    if (tc) NLF_CUDA(cudaFuncSetAttribute(k_update_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM));
     for (int j0 = 0; j0 < maxp; j0 += NB) {
         a.j0 = j0;
-        k_pivot<T><<<K, 256, 0, c->stream>>>(a);
+        k_pivot_f32<<<K, PIV_THREADS, 0, c->stream>>>(a, nullptr);
         k_panel<T><<<dim3((maxn + 3) / 4, K), 256, 0, c->stream>>>(a);
-        if constexpr (std::is_same<T, float>::value) {
-            if (tc) {
-                k_update_tc<<<dim3(ntc, ntc, K), TC_THREADS, TC_SMEM, c->stream>>>(a, p->d_flag.as<int>() + 2);
-                continue;
-            }
-        }
         k_update<T><<<dim3(nt, nt, K), 256, smu, c->stream>>>(a);
     }
     NLF_CUDA(cudaGetLastError());
@@ -701,7 +769,7 @@ template <typename T> void factor_ops(nlfeti_problem *p, OpPool<T> &pool) {
                                                pool.Sp.template as<T>(), p->d_sd.as<SubdomainDesc>());
         NLF_CUDA(cudaGetLastError());
         // phase 2: sweep all pivots of the pinned S~_k
-        run_sweeps<T>(p, pool.Sp.template as<T>(), soff, gdim, gld, gend, pool.scratch, p->opt.factor_tc == 1);
+        run_sweeps<T>(p, pool.Sp.template as<T>(), soff, gdim, gld, gend, pool.scratch, p->opt.factor_tc != 0);
         k_finish_inverse<T><<<g, 256, 0, c->stream>>>(pool.Sp.template as<T>(), p->d_sd.as<SubdomainDesc>());
         if (p->n_floating > 0) {
             DevMem V, C;

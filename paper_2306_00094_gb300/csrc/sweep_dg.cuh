@@ -661,17 +661,18 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_update_dg(DigitArgs a) {
 }
 
 // the lower triangle from the upper one, 32 x 32 tiles through shared memory; grid (tiles, tiles, K)
-__global__ void __launch_bounds__(256) k_mirror_up(double *pool, const int64_t *moff, const int32_t *mdim,
+template <typename T>
+__global__ void __launch_bounds__(256) k_mirror_up(T *pool, const int64_t *moff, const int32_t *mdim,
                                                    const int32_t *mld) {
     const int k = blockIdx.z, n = mdim[k], ld = mld[k];
     const int ti = blockIdx.y, tl = blockIdx.x;       // writes tile (rows ti, columns tl), tl <= ti
     if (ti * 32 >= n || tl > ti) return;
-    double *M = pool + moff[k];
-    __shared__ double t[32][33];
+    T *M = pool + moff[k];
+    __shared__ T t[32][33];
     const int x = threadIdx.x % 32, y0 = threadIdx.x / 32;
     for (int y = y0; y < 32; y += 8) {
         const int rr = tl * 32 + y, cc = ti * 32 + x;
-        t[y][x] = rr < n && cc < n ? M[(int64_t)rr * ld + cc] : 0.0;
+        t[y][x] = rr < n && cc < n ? M[(int64_t)rr * ld + cc] : T(0);
     }
     __syncthreads();
     for (int y = y0; y < 32; y += 8) {
