@@ -467,7 +467,7 @@ void run_sweeps_dg(nlfeti_problem *p, double *pool, const std::vector<int64_t> &
     }
     if (maxp == 0) return;
     const size_t tiles = (size_t)(rows / DG_TILE), dbytes = tiles * DG * DG_TBYTES;
-    const size_t need = 2 * dbytes + (size_t)K * DG * (DG_TBYTES / 2) + sizeof(double) * ((size_t)rows * NB + (size_t)K * NB * NB) +
+    const size_t need = 2 * dbytes + (size_t)K * DG * (DG_TBYTES / 2) + sizeof(double) * (size_t)K * NB * NB +
                         sizeof(int) * (2 * (size_t)rows + 2 * (size_t)K * NB);
     if (scratch.bytes < need) scratch.alloc(c, need);
     DevMem d_moff, d_mdim, d_mld, d_pend, d_soff;
@@ -481,8 +481,7 @@ void run_sweeps_dg(nlfeti_problem *p, double *pool, const std::vector<int64_t> &
     a.pan_d = scratch.as<unsigned char>();
     a.old_d = a.pan_d + dbytes;
     a.dinv_d = a.old_d + dbytes;
-    a.pan = reinterpret_cast<double *>(a.dinv_d + (size_t)K * DG * (DG_TBYTES / 2));
-    a.dinv = a.pan + rows * NB;
+    a.dinv = reinterpret_cast<double *>(a.dinv_d + (size_t)K * DG * (DG_TBYTES / 2));
     a.pan_e = reinterpret_cast<int *>(a.dinv + (size_t)K * NB * NB);
     a.old_e = a.pan_e + rows;
     a.dinv_e = a.old_e + rows;

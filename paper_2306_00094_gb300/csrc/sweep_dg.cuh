@@ -22,7 +22,7 @@
 //
 // Step over pivot block J (NB = 64 wide), three kernels: k_pivot_dg inverts the block (FP64, one CTA
 // per subdomain) and splits D^-1; k_panel_dg takes 128 rows of M_J, splits them (old), forms pan =
-// old D^-1 with the same digit products and splits pan; k_update_dg subtracts pan old^T.
+// old D^-1 with the same digit products, writes it to M and splits it; k_update_dg subtracts pan old^T.
 // M is symmetric, so the sweep keeps only its block upper triangle (128-wide blocks, the diagonal
 // ones whole) and k_mirror_up fills the rest at the end: half the products, half the traffic.  The
 // update's lanes are columns of M: its accesses are coalesced.
@@ -32,8 +32,9 @@
 // 128 x 64 x 16 per block.  An MMA of this shape takes about 61 clocks (as long with N = 32: reading A
 // sets its pace), so N = 64; seven accumulators of 64 columns fill tensor memory, so the high orders
 // (0 .. 3) and the low ones take turns: sixteen warps drain one part while the other is formed.  Per
-// block of 8192 entries 6.8 k clocks of MMA against 4.1 k of the FP64 pipe.  Measured on that row: 0.80 ms per
-// step (the MMAs alone 0.32), against 15.3 ms; factorization and one solve 422 -> 38 ms.
+// block of 8192 entries 6.8 k clocks of MMA against 4.1 k of the FP64 pipe.  The entries of J are written by k_panel_dg
+// (taken here, lane by lane, they cost 0.08 ms).  Measured on that row: 0.73 ms per step of the 36 matrices (the
+// MMAs alone 0.32), against 15.3 ms; factorization and one solve 422 -> 35.5 ms.
 // Every wait is bounded: one that runs out sets the sweep's timeout word; the CTA then waits (bounded)
 // for its copies and MMAs, frees its tensor memory and returns.
 #pragma once
@@ -53,7 +54,6 @@ constexpr int DG_CHUNK = 16;                        // blocks of a CTA
 
 struct DigitArgs {
     double *M;                // pool base
-    double *pan;              // per subdomain: n x NB
     double *dinv;             // per subdomain: NB x NB
     unsigned char *pan_d;     // digits of pan and old: per subdomain, per 128-row tile, DG x 16 KB
     unsigned char *old_d;
@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(DG_PAN_THREADS, 1) k_panel_dg(DigitArgs a) {
     const int n = a.mdim[k], ld = a.mld[k], tile = blockIdx.x, r0 = tile * DG_TILE;
     if (r0 >= n) return;
     const int b = min(NB, pend - a.j0), j0 = a.j0, jt = j0 / DG_TILE;
-    const double *M = a.M + a.moff[k];
+    double *M = a.M + a.moff[k];
     extern __shared__ __align__(1024) unsigned char dg_raw[];
     unsigned char *sa = dg_raw + ((1024u - (tc_s32(dg_raw) & 1023u)) & 1023u), *sb = sa + DG * DG_TBYTES;
     __shared__ uint64_t bar_b, bar_mma;
@@ -455,11 +455,20 @@ __global__ void __launch_bounds__(DG_PAN_THREADS, 1) k_panel_dg(DigitArgs a) {
     const int Ep = row_exp();
     split_rows(Ep);
     if (h == 0) a.pan_e[row0 + r] = Ep;
+    // M_iJ = pan (-D^-1 for the rows of J), where M_iJ was read; in the pivot's diagonal tile, which is
+    // whole, also the transposed entries of the other rows.  k_update_dg leaves J alone
     if (i < n) {
-        double *dst = a.pan + (row0 + r) * NB + 16 * h;
+        const int ij = i - j0;
+        const bool iJ = ij >= 0 && ij < b;
+        const double *D = a.dinv + (int64_t)k * NB * NB + (iJ ? ij : 0) * NB;
 #pragma unroll
-        for (int s = 0; s < 16; s += 2)
-            *reinterpret_cast<double2 *>(dst + s) = make_double2(dg_shift(x[s], -spc[16 * h + s]), dg_shift(x[s + 1], -spc[16 * h + s + 1]));
+        for (int s = 0; s < 16; ++s) {
+            const int c = 16 * h + s;
+            if (c >= b) continue;
+            const double v = dg_shift(x[s], -spc[c]);
+            if (tile <= jt) M[(int64_t)i * ld + j0 + c] = iJ ? -D[c] : v;
+            if (tile >= jt && !iJ) M[(int64_t)(j0 + c) * ld + i] = v;
+        }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -574,7 +583,6 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_update_dg(DigitArgs a) {
         const int i = c0 + 32 * qd + lane;
         const bool in = i < n, iJ = i >= j0 && i < j1;
         const int Ea = in ? a.pan_e[row0 + i] : 0;
-        const double *pan = a.pan + row0 * NB, *D = a.dinv + (int64_t)k * NB * NB;
         const uint32_t ta = tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(16 * hf);
         for (int q = q0; q < q1; ++q) {
             const int ph = (q - q0) & 1, l0 = q * DG_LB + 16 * hf;
@@ -637,16 +645,10 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_update_dg(DigitArgs a) {
                 }
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
-                    double o = m[cc + c] - dg_value(hi[cc + c], dg_lo(acc, c), Ea + eo[c]);
-                    if (!plain) {
-                        const int l = l0 + cc + c;
-                        if (!in || l >= n) continue;
-                        const bool lJ = l >= j0 && l < j1;
-                        if (iJ && lJ) o = -D[(i - j0) * NB + (l - j0)];
-                        else if (lJ) o = pan[(int64_t)i * NB + (l - j0)];
-                        else if (iJ) o = pan[(int64_t)l * NB + (i - j0)];
-                    }
-                    Mp[(int64_t)(cc + c) * ld] = o;
+                    const double o = m[cc + c] - dg_value(hi[cc + c], dg_lo(acc, c), Ea + eo[c]);
+                    const int l = l0 + cc + c;       // J holds its new values already
+                    if (plain || (in && !iJ && l < n && (l < j0 || l >= j1)))
+                        Mp[(int64_t)(cc + c) * ld] = o;
                 }
             }
         }
