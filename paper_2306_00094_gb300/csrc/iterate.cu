@@ -3,8 +3,8 @@
 // iterative refinement on the torn system (eq. discreteKKT).
 //
 // Vectors hold R right-hand sides interleaved (entry i of column c at i*R + c).
-// Lambda-space vectors, coarse vectors and all scalars are FP64; the subdomain operators
-// S_k^+, S_k and the swept matrices are FP64 (plain path) or FP32 (mixed path).
+// The subdomain operators S_k^+, S_k and the swept matrices are FP64 (plain path) or FP32 (mixed
+// path), the PCG's Lambda-space vectors likewise; a pass's set-up and exit, the scalars and the refinement are FP64.
 //
 // PCG iteration (per right-hand side; converged columns are frozen with eta = 0):
 //   w = P r;  z = B_D S B_D^T w;  y = P z;  beta = (y,w)/(y,w)_old;  p = y + beta p;
@@ -1601,9 +1601,11 @@ struct Runner {
         gate = nullptr;
     }
 
-    // One PCG iteration, ten kernels.  The updates of p, lambda and r are stored by the next
-    // iteration's k_check_update (kernels before it form p_new and r_new per row), and
-    // k_check_update sets the loop condition inside a graph loop.  The Lambda vectors and their
+    // One PCG iteration: four kernels with the Lambda steps in clusters (iteration_clusters), else ten
+    // (iteration_rows).  The updates of p, lambda and r are stored by the next iteration's first kernel
+    // (kernels before it form p_new and r_new per row), whose stop test sets the loop condition
+    // inside a graph loop (on a branch of the body beside the next kernels it made FP64 solves 2 to 8 %
+    // slower).  The Lambda vectors and their
     // arithmetic are in the operators' type T: FP64 in the FP64 pass; FP32 in the FP32 pass,
     // whose iterations only have to reduce the residual by inner_tol (the refinement's FP64
     // residual corrects what FP32 leaves).  The dot products' tile sums and the PCG scalars are

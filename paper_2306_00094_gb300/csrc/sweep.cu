@@ -15,8 +15,8 @@
 // Pivot blocks are NB = 64 wide; a step is three launches over all subdomains: invert
 // the pivot block (one CTA per subdomain), form the pivot panels, update all tiles.  FP64: on the
 // tensor cores by exact digit products, block upper triangle only (sweep_dg.cuh).  FP32: likewise
-// (sweep_d4.cuh), or with factor_tc = 0 64x64 CTA tiles, 4x4 register blocking, on the FP32 pipes.  A non-positive pivot sets the device status word (NLFETI_E_NOT_SPD)
-// instead of trapping.
+// (sweep_d4.cuh), or with factor_tc = 0 64x64 CTA tiles, 4x4 register blocking, on the FP32 pipes.
+// A non-positive pivot sets the device status word (NLFETI_E_NOT_SPD) instead of trapping.
 #include <algorithm>
 #include <numeric>
 #include <type_traits>
