@@ -603,7 +603,8 @@ __global__ void __launch_bounds__(256) k_coarse_solve(const double *gpart, int p
 // order).  Blocks take chunks of up to RED_THREADS columns (grid y), a thread one column of every
 // (threads / chunk)-th row, so that neighbouring threads read neighbouring entries; a block's maxima are combined
 // per column in shared memory and the last block to arrive writes corr.  (One block row per column,
-// each reading every R-th entry, took 80 us on the peridynamic workload, 168200 x 16; now 12 us on the factorization workload, 36450 x 2, from 23.)
+// each reading every R-th entry, took 80 us on the peridynamic workload with 16 columns; now 38, and 12 instead of
+// 23 us with two columns of 36450 entries.)
 inline dim3 refine_grid(int64_t n, int R) {
     const int cb = std::min(R, RED_THREADS), rows = RED_THREADS / cb;
     return dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>(RED_BLOCKS, (n + rows - 1) / rows)), (R + cb - 1) / cb);
