@@ -752,20 +752,25 @@ __global__ void __launch_bounds__(RED_THREADS) k_cg_init(const double *b, const 
 // Each slot's sum runs over its nonzeros in order, the slots are summed by two shuffles, and a
 // unit's 32 products p q by one warp tree per column, so a column's arithmetic is the same
 // whatever R.
+// With 8 columns a CTA has 8 warps of 4 rows each in turn: 32 warps of one row and two barriers per unit left
+// the SM to one CTA, idle at every barrier (const l2, 21000 dofs, 8 columns, the whole CG: 14.7 ms, now 13.1).
+__host__ __device__ constexpr int cg_spmv_threads(int cw) { return cw == 8 ? 256 : 128 * cw; }
 template <int CW>
-__global__ void __launch_bounds__(128 * CW) k_cg_spmv(const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
+__global__ void __launch_bounds__(cg_spmv_threads(CW), CW == 8 ? 4 : 1) k_cg_spmv(const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
                                                       const float *__restrict__ vhi, const float *__restrict__ vlo,
                                                       const float *__restrict__ ph, const float *__restrict__ pl,
                                                       const double *__restrict__ p, double *__restrict__ q, int64_t n,
                                                       int R, double *part, PcgScalars s) {
-    constexpr int NW = 4 * CW, RP = 8 / CW;       // warps, rows of a warp
+    constexpr int NW = cg_spmv_threads(CW) / 32, RP = 8 / CW;       // warps, rows of a warp at a time
     constexpr int NC = CW == 8 ? CG_MAX_R : CW;
     __shared__ double prods[CG_UNIT][NC + 1], dsum[NC];
     if (*s.n_active == 0) return;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, kg = lane >> 3;
-    const int cl = lane & (CW - 1), row = warp * RP + (lane & 7) / CW;
+    const int cl = lane & (CW - 1);
     if (threadIdx.x < NC) dsum[threadIdx.x] = 0.0;
     for (int64_t i0 = (int64_t)blockIdx.x * CG_UNIT; i0 < n; i0 += (int64_t)gridDim.x * CG_UNIT) {
+#pragma unroll 1
+        for (int row = warp * RP + (lane & 7) / CW; row < CG_UNIT; row += NW * RP) {
         const int64_t i = i0 + row;
         const int64_t a = i < n ? ptr[i] : 0, e = i < n ? ptr[i + 1] : 0;
         for (int c0 = 0; c0 < R; c0 += 8) {
@@ -813,6 +818,7 @@ __global__ void __launch_bounds__(128 * CW) k_cg_spmv(const int64_t *__restrict_
                 prods[row][c] = on ? p[i * R + c] * acc : 0.0;
                 if (on) q[i * R + c] = acc;
             }
+        }
         }
         __syncthreads();
         for (int c = warp; c < R; c += NW) {
@@ -1723,7 +1729,7 @@ struct Runner {
         const unsigned blocks =
             (unsigned)std::max<int64_t>(1, std::min<int64_t>(CG_BLOCKS, (n + CG_UNIT - 1) / CG_UNIT));
         auto spmv = [&](auto kern, int cw) {
-            kern<<<blocks, 128 * cw, 0, st>>>(p->d_cg_ptr.as<int64_t>(), p->d_cg_col.as<int32_t>(),
+            kern<<<blocks, cg_spmv_threads(cw), 0, st>>>(p->d_cg_ptr.as<int64_t>(), p->d_cg_col.as<int32_t>(),
                                               p->d_cg_vhi.as<float>(), p->d_cg_vlo.as<float>(), ws.cg_ph.as<float>(),
                                               ws.cg_pl.as<float>(), pv, q, n, R, ws.cg_part.as<double>(), S);
         };
