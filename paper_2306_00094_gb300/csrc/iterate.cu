@@ -753,15 +753,17 @@ __global__ void __launch_bounds__(RED_THREADS) k_cg_init(const double *b, const 
 // unit's 32 products p q by one warp tree per column, so a column's arithmetic is the same
 // whatever R.
 // With 8 columns a CTA has 8 warps of 4 rows each in turn: 32 warps of one row and two barriers per unit left
-// the SM to one CTA, idle at every barrier (const l2, 21000 dofs, 8 columns, the whole CG: 14.7 ms, now 13.1).
+// the SM to one CTA, idle at every barrier (const l2, 21000 dofs, 8 columns, the whole CG: 14.7 ms, then 13.1; with four
+// loads per slot, so that six CTAs fit an SM, 12.1).
 __host__ __device__ constexpr int cg_spmv_threads(int cw) { return cw == 8 ? 256 : 128 * cw; }
 template <int CW>
-__global__ void __launch_bounds__(cg_spmv_threads(CW), CW == 8 ? 4 : 1) k_cg_spmv(const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
+__global__ void __launch_bounds__(cg_spmv_threads(CW), CW == 8 ? 6 : 1) k_cg_spmv(const int64_t *__restrict__ ptr, const int32_t *__restrict__ col,
                                                       const float *__restrict__ vhi, const float *__restrict__ vlo,
                                                       const float *__restrict__ ph, const float *__restrict__ pl,
                                                       const double *__restrict__ p, double *__restrict__ q, int64_t n,
                                                       int R, double *part, PcgScalars s) {
     constexpr int NW = cg_spmv_threads(CW) / 32, RP = 8 / CW;       // warps, rows of a warp at a time
+    constexpr int U = CW == 8 ? 4 : CG_U;         // nonzeros per slot loaded at a time
     constexpr int NC = CW == 8 ? CG_MAX_R : CW;
     __shared__ double prods[CG_UNIT][NC + 1], dsum[NC];
     if (*s.n_active == 0) return;
@@ -777,28 +779,28 @@ __global__ void __launch_bounds__(cg_spmv_threads(CW), CW == 8 ? 4 : 1) k_cg_spm
             const int c = c0 + cl;
             const bool on = c < R && i < n;
             float sh = 0.f, sl = 0.f;
-            // CG_U nonzeros per slot at a time: their matrix loads first, then their p gathers,
+            // U nonzeros per slot at a time: their matrix loads first, then their p gathers,
             // then the products in order (loads in flight cover the latency)
-            for (int64_t k0 = a + kg; k0 < e; k0 += 4 * CG_U) {
-                float ahv[CG_U], alv[CG_U];
-                int jv[CG_U];
+            for (int64_t k0 = a + kg; k0 < e; k0 += 4 * U) {
+                float ahv[U], alv[U];
+                int jv[U];
 #pragma unroll
-                for (int u = 0; u < CG_U; ++u) {
+                for (int u = 0; u < U; ++u) {
                     const int64_t k = k0 + 4 * u;
                     const bool in = k < e;
                     ahv[u] = in ? __ldg(vhi + k) : 0.f;
                     alv[u] = in ? __ldg(vlo + k) : 0.f;
                     jv[u] = in ? __ldg(col + k) : -1;
                 }
-                float xhv[CG_U], xlv[CG_U];
+                float xhv[U], xlv[U];
 #pragma unroll
-                for (int u = 0; u < CG_U; ++u) {
+                for (int u = 0; u < U; ++u) {
                     const bool in = on && jv[u] >= 0;
                     xhv[u] = in ? __ldg(ph + (int64_t)jv[u] * R + c) : 0.f;
                     xlv[u] = in ? __ldg(pl + (int64_t)jv[u] * R + c) : 0.f;
                 }
 #pragma unroll
-                for (int u = 0; u < CG_U; ++u) {
+                for (int u = 0; u < U; ++u) {
                     if (!on || jv[u] < 0) continue;
                     const float ah = ahv[u], al = alv[u], xh = xhv[u], xl = xlv[u];
                     // explicit round-to-nearest intrinsics: no contraction into fma
