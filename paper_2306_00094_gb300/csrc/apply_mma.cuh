@@ -314,6 +314,7 @@ __global__ void __launch_bounds__(MMA_THREADS, 1)
             const int64_t yoff = sd[k].offU;
 #pragma unroll
             for (int c0 = 0; c0 < NP; c0 += 16) {
+                __syncwarp();                       // the stores branch; the loads are .aligned
                 float v[16], t[16];
                 const uint32_t ta = tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)((j & 1) * MMA_ACC * NP + c0);
                 tc_ld16(ta, v);

@@ -445,6 +445,7 @@ __global__ void __launch_bounds__(D4_THREADS, 1) k_update_d4(Digit4Args a) {
             const uint32_t ta = tmem + ((uint32_t)(32 * qd) << 16) + (uint32_t)(ab * D4_ACC + (h & 1) * DG_LB + 32 * hf);
 #pragma unroll
             for (int cc = 0; cc < 32; cc += 8) {
+                __syncwarp();                       // the half block before branched at its stores; the loads are .aligned
                 uint32_t a0[8], a1[8];
                 dg_ld8(ta + (uint32_t)cc, a0);
                 dg_ld8(ta + (uint32_t)(DG_TILE + cc), a1);

@@ -440,6 +440,7 @@ __global__ void __launch_bounds__(DG_PAN_THREADS, 1) k_panel_dg(DigitArgs a) {
     // (scaled) pan = old D^-1: lane quarter warp mod 4 and columns 16 (warp / 4) .. are the thread's own
 #pragma unroll
     for (int c0 = 0; c0 < 16; c0 += 8) {
+        __syncwarp();                                // dg_value branches; the loads are .aligned
         uint32_t hi[DG_HI][8], lo[DG - DG_HI][8];
         const uint32_t ta = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(16 * h + c0);
 #pragma unroll
@@ -479,8 +480,10 @@ __global__ void __launch_bounds__(DG_PAN_THREADS, 1) k_panel_dg(DigitArgs a) {
         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
-    if (warp == 0)
+    if (warp == 0) {
+        __syncwarp();                                // lane 0 waited for its copies
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    }
 }
 
 // grid (column tiles of the largest subdomain, last first; chunks of DG_CHUNK row blocks; K)
@@ -610,6 +613,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_update_dg(DigitArgs a) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
             for (int cc = 0; cc < 16; cc += 4) {
+                __syncwarp();                        // the loads are .aligned
                 uint32_t acc[DG_HI][4];
 #pragma unroll
                 for (int d = 0; d < DG_HI; ++d) dg_ld4(ta + (uint32_t)(d * DG_LB + cc), acc[d]);
@@ -633,6 +637,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_update_dg(DigitArgs a) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
             for (int cc = 0; cc < 16; cc += 4) {
+                __syncwarp();                        // dg_value and the stores branch
                 uint32_t acc[DG - DG_HI][4];
 #pragma unroll
                 for (int d = DG_HI; d < DG; ++d) dg_ld4(ta + (uint32_t)(d * DG_LB + cc), acc[d - DG_HI]);
