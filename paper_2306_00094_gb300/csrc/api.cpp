@@ -491,20 +491,22 @@ namespace nlf {
 // the sweep scratch and the node maps, plus a margin for the index maps and tensor maps.
 size_t problem_bytes(const Decomp &d, int64_t n_nodes, int mask) {
     const int K = d.K, nc = d.nc;
-    double b = 0, sum_nk = 0;
+    double b = 0, sum_nk = 0, rows = 0;
     for (int k = 0; k < K; ++k) {
         const double nk = (double)d.nodes[k].size() * nc, nG = (double)d.n_gamma_nodes[k] * nc;
         const double nD = (double)d.dir_nodes[k].size() * nc;
         const double ldM = (double)round8((int)nk), ldG = (double)round8(std::max((int)nG, 1));
         sum_nk += nk;
+        rows += std::ceil(nk / 128) * 128;                                // of the sweeps' panels
         b += 8.0 * nk * nk + 8.0 * nk * nD;                               // A^k and its Dirichlet block
         if (mask & 1) b += 8.0 * nk * ldM + 2 * 8.0 * nG * ldG;           // FP64 swept matrix, S, S^+
         if (mask & 2) b += 4.0 * nk * ldM * 3 + 2 * 4.0 * nG * ldG + 2.0 * nG * ldG;   // FP32 + A pairs, S, S^+, FP16 S
     }
-    const double scr = sum_nk * 64 * 2 + (double)K * 64 * 64;              // sweep panels
-    // FP64: the panel and its digits and those of the pivot rows, rows padded to 128
-    if (mask & 1) b += (sum_nk + 128.0 * K) * (512 + 1792 + 8) + (double)K * (32768 + 57344 + 512);
-    if (mask & 2) b += 4.0 * scr;
+    // scratch of the sweeps: the digits of the panel and of the pivot rows (FP64: 2 x 7 of 128 bytes a
+    // row, FP32: 2 x 4) and a scale of each; per subdomain the inverted pivot block, its digits (FP64)
+    // and the exponents of the pivots
+    if (mask & 1) b += rows * (1792 + 8) + (double)K * (32768 + 57344 + 512);
+    if (mask & 2) b += rows * (1024 + 8) + (double)K * (16384 + 256);
     b += 4.0 * (double)K * (double)n_nodes;                               // node -> subdomain-local maps
     b += 64.0 * sum_nk;                                                   // index maps, vectors, tensor maps
     // (G^T G)^-1 in FP64 and its FP32 copy, at most every subdomain floating (1 kernel vector
