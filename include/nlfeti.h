@@ -244,7 +244,8 @@ nlfeti_status nlfeti_problem_set_matrix(nlfeti_problem *p, int k, const double *
  * over the operator (1, 2, 4, 8 or 16, at most nrhs; 8 for FP64: fewer passes read the operator
  * fewer times but hold more accumulators), ctas_per_sm (1 or 2) of its persistent grid, and
  * rows_per_warp (4, or 8 for the FP32 and FP16 operators with rc >= 4: half the consumer warps,
- * each shared-memory load of x serving twice the rows).
+ * each shared-memory load of x serving twice the rows).  The default: the smallest block that holds
+ * all nrhs (at most the widest), two CTAs per SM, and 4 rows per warp, 8 with a block of 16.
  * nlfeti_autotune times every candidate with CUDA events on the problem's factored operators
  * for each operator kind it has -- 0 FP32 S_k^+ and S_k, 1 the FP16 copy of S_k the mixed
  * path's preconditioner applies, 2 FP64 -- and keeps the fastest in the problem: later solves
@@ -258,9 +259,12 @@ nlfeti_status nlfeti_problem_set_matrix(nlfeti_problem *p, int k, const double *
  * gives bitwise the same results (each column is summed in the same order whatever the pass
  * width and schedule); the tensor-core preconditioner rounds differently (it only steers the
  * PCG: the iteration count may change, not the accuracy reached).
- * nlfeti_set_apply_choice pins a shape (rc 0 clears it, back to the default: the widest block
- * up to nrhs, two CTAs per SM, 4 rows per warp; rc -1 selects the tensor-core apply for kind 1;
- * rows_per_warp 0 means 4);
+ * Between two block sizes the default's block is wider than nrhs, which no choice can name: the
+ * tuner times it and reports it in the place of the widest block up to nrhs with two CTAs per SM
+ * and 4 rows per warp, which needs a second pass over the operator (in the cache file it has
+ * rc 0).  Entries of cache files written with another set of shapes are not used.
+ * nlfeti_set_apply_choice pins a shape, which then runs as named (rc 0 clears it, back to the
+ * default; rc -1 selects the tensor-core apply for kind 1; rows_per_warp 0 means 4);
  * NLFETI_E_INVALID for shapes outside the lists above. */
 typedef struct {
     int32_t kind, nrhs, rc, ctas_per_sm;

@@ -52,7 +52,7 @@ constexpr int APPLY_NS_H16 = 3;                     // ... at RC = 16 (32 KB eac
 __host__ __device__ constexpr int apply_rc(int R, int elem_size) {
     return (R > 8 && elem_size == 4) ? 16 : (R > 4 ? 8 : (R > 2 ? 4 : (R > 1 ? 2 : 1)));
 }
-// the widest block of at most R columns (what the tuner's choices name)
+// the widest block of at most R columns
 __host__ __device__ constexpr int apply_rc_below(int R, int elem_size) {
     return (R >= 16 && elem_size == 4) ? 16 : (R >= 8 ? 8 : (R >= 4 ? 4 : (R >= 2 ? 2 : 1)));
 }

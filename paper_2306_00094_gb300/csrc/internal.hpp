@@ -195,8 +195,8 @@ template <typename T> struct OpPool {   // operators of one precision
 namespace nlf { struct SolveWS; }
 
 // a configuration of the bulk-copy interface apply: right-hand sides per streamed pass (1, 2,
-// 4, 8 or 16) and CTAs per SM of its persistent grid (1 or 2); for the FP16 copy of S_k the
-// tensor-core apply instead (mma)
+// 4, 8 or 16; 0 = the default shape) and CTAs per SM of its persistent grid (1 or 2); for the FP16
+// copy of S_k the tensor-core apply instead (mma)
 struct ApplyChoice {
     int rc = 0;
     int per_sm = 2;
@@ -331,7 +331,7 @@ void stream_leave(nlfeti_ctx *c);
 void ctx_attach(nlfeti_ctx *c);
 void ctx_detach(nlfeti_ctx *c);
 // the apply configuration used for operator kind (0 FP32, 1 FP16 copy, 2 FP64) and R: the
-// autotuner's choice if one was made, else the default (apply_rc(R), two CTAs per SM)
+// autotuner's or the caller's choice if one was made, else the default (rc = 0)
 ApplyChoice apply_choice(const nlfeti_problem *p, int kind, int R);
 // streaming multiprocessors of the current device
 int device_sms();

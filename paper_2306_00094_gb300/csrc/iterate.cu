@@ -1272,11 +1272,10 @@ struct Runner {
 
 
     template <typename T> int apply_tma(const OpPool<T> &pool, int use_sp, double *y, bool half = false) {
-        // the autotuner's choice for this operator kind and R (column block, CTAs per SM), else
-        // the default block and two CTAs per SM
+        // the shape chosen for this operator kind and R (column block, CTAs per SM, rows per warp), else
+        // the default: the block that holds all R and two CTAs per SM
         const ApplyChoice ch = apply_choice(p, half ? 1 : (sizeof(T) == 8 ? 2 : 0), R);
-        // (the default shape named by its widest block up to R runs as the default)
-        const bool dflt = ch.rc <= 0 || (ch.rc == apply_rc_below(R, (int)sizeof(T)) && ch.per_sm == 2 && ch.rpw == 4);
+        const bool dflt = ch.rc <= 0;
         const int rc = dflt ? apply_rc(R, (int)sizeof(T)) : ch.rc;
         const int ri = rc >= 16 ? 4 : (rc >= 8 ? 3 : (rc >= 4 ? 2 : (rc >= 2 ? 1 : 0)));
         const CUtensorMap *xm = ws.xmaps_rc[sizeof(T) == 8 ? 1 : 0][ri].template as<CUtensorMap>();
@@ -1324,7 +1323,7 @@ struct Runner {
                   }
                 }
                 // sixteen columns with two CTAs per SM: eight rows per warp and no producer warp (the
-                // default; four rows only when the tuner or the caller names them beside another block)
+                // default; four rows when they are chosen)
                 if constexpr (RCT == 16) {
                     if (dflt || ch.rpw == 8) {
                         auto self = [&](auto ns_tag, auto mt_tag) {
@@ -2314,11 +2313,7 @@ void solve_device(nlfeti_problem *p, SolveWS &ws, cudaStream_t st, int R, int rh
 
 ApplyChoice apply_choice(const nlfeti_problem *p, int kind, int R) {
     auto it = p->tune.find({kind, R});
-    if (it != p->tune.end()) return it->second;
-    ApplyChoice c;
-    c.rc = apply_rc_below(R, kind == 2 ? 8 : 4);
-    c.per_sm = 2;
-    return c;
+    return it != p->tune.end() ? it->second : ApplyChoice{};
 }
 
 int device_sms() {
@@ -2330,13 +2325,15 @@ int device_sms() {
 
 namespace {
 
-// key of a tuning result: the device, the subdomain operator shapes, the kind and R
+// key of a tuning result: the set of shapes, the device, the subdomain operator shapes, the kind and R
 std::string tune_key(const nlfeti_problem *p, int kind, int R) {
     uint64_t h = 1469598103934665603ull;
     auto mix = [&](const void *q, size_t n) {
         const unsigned char *b = static_cast<const unsigned char *>(q);
         for (size_t i = 0; i < n; ++i) { h ^= b[i]; h *= 1099511628211ull; }
     };
+    const int shapes = 2;            // a new number when a shape's name gets another kernel: old timings don't count
+    mix(&shapes, sizeof(shapes));
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceProp prop{};
@@ -2360,7 +2357,7 @@ struct CacheLine {
     double us = 0;
 };
 
-// the cache: {"entries": [ one object per line ]}
+// the cache: {"entries": [ one object per line ]}; rc = 0 is the default shape, where it has no name
 std::vector<CacheLine> read_tune_cache(const char *path) {
     std::vector<CacheLine> out;
     FILE *f = path ? fopen(path, "r") : nullptr;
@@ -2413,6 +2410,18 @@ void autotune_applies(nlfeti_problem *p, int R, const char *cache_path, std::vec
     const int saved_batched = p->opt.batched, saved_fp16 = p->opt.precond_fp16;
     p->opt.batched = 1;
     bool changed = false;
+    // the default takes a block wider than R between two block sizes.  No choice can name that shape: it is
+    // timed and reported in the place of the widest block up to R with two CTAs and 4 rows, whose second
+    // pass over the operator it saves
+    const auto unnamed_default = [&](int kind, int rc, int per_sm, int rpw) {
+        const int es = kind == 2 ? 8 : 4;
+        return apply_rc(R, es) > R && rc == apply_rc_below(R, es) && per_sm == 2 && rpw == 4;
+    };
+    const auto choose = [&](const TuneEntry &te) {
+        if (te.rc == -1) p->tune[{te.kind, R}] = ApplyChoice{0, 2, 1};
+        else if (unnamed_default(te.kind, te.rc, te.per_sm, te.rpw)) p->tune.erase({te.kind, R});
+        else p->tune[{te.kind, R}] = ApplyChoice{te.rc, te.per_sm, 0, te.rpw};
+    };
     cudaEvent_t ea = nullptr, eb = nullptr;
     NLF_CUDA(cudaEventCreate(&ea));
     NLF_CUDA(cudaEventCreate(&eb));
@@ -2428,7 +2437,7 @@ void autotune_applies(nlfeti_problem *p, int R, const char *cache_path, std::vec
             const std::string key = tune_key(p, kind, R);
             for (const auto &c : cache)
                 if (c.key == key && c.kind == kind && c.R == R) {
-                    te.rc = c.rc;
+                    te.rc = c.rc == 0 ? apply_rc_below(R, kind == 2 ? 8 : 4) : c.rc;
                     te.per_sm = c.per_sm;
                     te.rpw = c.rpw;
                     te.us = c.us;
@@ -2444,7 +2453,11 @@ void autotune_applies(nlfeti_problem *p, int R, const char *cache_path, std::vec
                     for (int rpw = 4; rpw <= 8; rpw += 4) {
                         // eight rows per warp: the FP32 and FP16 operators, four or more columns
                         if (rpw == 8 && (kind == 2 || rc < 4)) continue;
-                        p->tune[{kind, R}] = ApplyChoice{rc, per_sm, 0, rpw};
+                        TuneEntry cand = te;
+                        cand.rc = rc;
+                        cand.per_sm = per_sm;
+                        cand.rpw = rpw;
+                        choose(cand);
                         auto launch = [&] {
                             if (kind == 0) run.symv<float>(p->op32, 1, ws.xP.as<float>(), ws.yU.as<double>());
                             else if (kind == 1) run.symv<float>(p->op32, 0, ws.xP.as<float>(), ws.yU.as<double>(), true);
@@ -2457,13 +2470,10 @@ void autotune_applies(nlfeti_problem *p, int R, const char *cache_path, std::vec
                         NLF_CUDA(cudaEventSynchronize(eb));
                         float ms = 0.f;
                         NLF_CUDA(cudaEventElapsedTime(&ms, ea, eb));
-                        const double us = 1e3 * ms / 3.0;
-                        if (us < best) {
-                            best = us;
-                            te.rc = rc;
-                            te.per_sm = per_sm;
-                            te.rpw = rpw;
-                            te.us = us;
+                        cand.us = 1e3 * ms / 3.0;
+                        if (cand.us < best) {
+                            best = cand.us;
+                            te = cand;
                         }
                     }
                 }
@@ -2494,19 +2504,15 @@ void autotune_applies(nlfeti_problem *p, int R, const char *cache_path, std::vec
                 c.key = key;
                 c.kind = kind;
                 c.R = R;
-                c.rc = te.rc;
+                c.rc = te.rc != -1 && unnamed_default(kind, te.rc, te.per_sm, te.rpw) ? 0 : te.rc;
                 c.per_sm = te.per_sm;
                 c.rpw = te.rpw;
                 c.us = te.us;
                 cache.push_back(c);
                 changed = true;
             }
-            if (te.rc == -1) {
-                build_tiled_half(p);
-                p->tune[{kind, R}] = ApplyChoice{apply_rc_below(R, 4), 2, 1};
-            } else {
-                p->tune[{kind, R}] = ApplyChoice{te.rc, te.per_sm, 0, te.rpw};
-            }
+            if (te.rc == -1) build_tiled_half(p);
+            choose(te);
             out.push_back(te);
         }
     } catch (...) {

@@ -80,8 +80,8 @@ void apply_operator(nlfeti_problem *p, SolveWS &ws, cudaStream_t st, int op, int
 
 // Autotuner of the bulk-copy interface apply for R right-hand sides: per operator kind the
 // problem has (FP32 S^+, FP16 copy of S_k, FP64 S^+), every column block 1..16 (<= R) and one or
-// two CTAs per SM, timed with CUDA events on the problem's operators; the fastest is kept in
-// the problem.  With a cache path, choices found there (same device, subdomain shapes, kind and
+// two CTAs per SM, and the default where its block is wider, timed with CUDA events on the problem's
+// operators; the fastest is kept in the problem.  With a cache path, choices found there (same device, subdomain shapes, kind and
 // R) are used without timing, and new ones are written back (JSON).
 struct TuneEntry {
     int kind = 0, R = 0, rc = 0, per_sm = 0, rpw = 4;
