@@ -116,9 +116,10 @@ typedef struct {
  *          nlfeti_apply ops 0-4 always use the FP32 S_k.
  * factor_tc (FP32 operators): the rank-64 updates of the factorization sweeps on the tensor
  *          cores (tcgen05 kind::f16 on BF16 digits of the FP32 panels, the leading products exact) --
- *          2 (the default) and 1 = in both sweeps (the Omega sweep of A^k and the sweep of the pinned
- *          S_k), 0 = on the FP32 pipes only.  The digit products round less than a dot product on the FP32
- *          pipes; all settings meet the same tolerances.  Read by nlfeti_factor.
+ *          1 = in both sweeps (the Omega sweep of A^k and the sweep of the pinned S_k; the
+ *          default), 2 = in the Omega sweep only, 0 = on the FP32 pipes only.  The digit products
+ *          round less than a dot product on the FP32 pipes, but keep 35 bits below the largest
+ *          entry of a panel row; all settings meet the same tolerances.  Read by nlfeti_factor.
  * residual_format (mixed path): how the FP32 factorization keeps A^k for the FP64-accurate
  *          refinement residual (double-single arithmetic either way) -- 0 = chosen from the
  *          sparsity of A^k (the default): a CSR when at most an eighth of the dense entries are

@@ -404,7 +404,7 @@ void nlfeti_default_options(nlfeti_options *o) {
     o->hbm_budget = 0;
     o->graph_loop = 1;
     o->precond_fp16 = 1;
-    o->factor_tc = 2;
+    o->factor_tc = 1;
     o->residual_format = 0;
 }
 

@@ -15,7 +15,8 @@
 // Pivot blocks are NB = 64 wide; a step is three launches over all subdomains: invert
 // the pivot block (one CTA per subdomain), form the pivot panels, update all tiles.  FP64: on the
 // tensor cores by exact digit products, block upper triangle only (sweep_dg.cuh).  FP32: likewise
-// (sweep_d4.cuh), or with factor_tc = 0 64x64 CTA tiles, 4x4 register blocking, on the FP32 pipes.
+// (sweep_d4.cuh), or in the sweeps that factor_tc leaves out 64x64 CTA tiles, 4x4 register blocking, on
+// the FP32 pipes.
 // A non-positive pivot sets the device status word (NLFETI_E_NOT_SPD) instead of trapping.
 #include <algorithm>
 #include <numeric>
@@ -768,7 +769,7 @@ template <typename T> void factor_ops(nlfeti_problem *p, OpPool<T> &pool) {
                                                pool.Sp.template as<T>(), p->d_sd.as<SubdomainDesc>());
         NLF_CUDA(cudaGetLastError());
         // phase 2: sweep all pivots of the pinned S~_k
-        run_sweeps<T>(p, pool.Sp.template as<T>(), soff, gdim, gld, gend, pool.scratch, p->opt.factor_tc != 0);
+        run_sweeps<T>(p, pool.Sp.template as<T>(), soff, gdim, gld, gend, pool.scratch, p->opt.factor_tc == 1);
         k_finish_inverse<T><<<g, 256, 0, c->stream>>>(pool.Sp.template as<T>(), p->d_sd.as<SubdomainDesc>());
         if (p->n_floating > 0) {
             DevMem V, C;
