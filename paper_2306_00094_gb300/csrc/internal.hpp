@@ -318,7 +318,14 @@ template <typename T> void factor_ops(nlfeti_problem *p, OpPool<T> &pool);
 void build_tiled_half(nlfeti_problem *p);
 void setup_coarse(nlfeti_problem *p);
 void setup_jump_weights(nlfeti_problem *p);
-// the Lambda-space operators in the form the PCG iterations read (after the two above)
+// whether the Lambda rows, the U dofs and the places of the U dofs in the apply inputs (column layout n_up,
+// paired layout n_xp entries per right-hand side) can be told by the 32-bit indices of the Lambda-space
+// operators; a signed row of B^T is its number plus one
+inline bool lambda_indices_fit(int64_t n_lambda, int64_t n_u, int64_t n_up, int64_t n_xp) {
+    return n_lambda < INT32_MAX && n_u <= INT32_MAX && n_up <= INT32_MAX && n_xp <= INT32_MAX;
+}
+// the Lambda-space operators in the form the PCG iterations read (after the two above); fails where
+// their indices do not fit
 void setup_lambda(nlfeti_problem *p);
 // whether the cluster kernels run this problem: sizes within their limits and clusters of their
 // size schedulable on the device (sets the kernels' attributes)

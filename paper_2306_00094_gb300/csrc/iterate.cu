@@ -2747,7 +2747,6 @@ int apply_mma_ctas() {
 
 bool lambda_clusters_ok(const nlfeti_problem *p, int bd_w) {
     if (p->n_lambda < 1 || p->n_lambda > LAM_MAX_ROWS || p->n_co > LAM_MAX_CO || bd_w > LAM_MAX_ELL) return false;
-    if (p->n_xp > INT32_MAX || p->n_up > INT32_MAX || p->n_lambda * LAM_MAX_ELL > INT32_MAX) return false;
     const size_t smem = std::max(lam_smem_bytes<double, 2>(p->n_co, p->n_floating),
                                  lam_smem_bytes<float, 4>(p->n_co, p->n_floating));
     if (smem > LAM_MAX_SMEM) return false;

@@ -1187,6 +1187,8 @@ __global__ void k_flip(const int32_t *ai, const double *av, int64_t n, int w, in
 void setup_lambda(nlfeti_problem *p) {
     nlfeti_ctx *c = p->ctx;
     const int64_t nl = p->n_lambda, nu = p->n_u;
+    if (!lambda_indices_fit(nl, nu, p->n_up, p->n_xp))
+        fail(NLFETI_E_INVALID, "the interface has more than 2^31 - 1 dofs or apply input entries");
     int zmax = 0;                    // most copies of a node: entries of a B_D row (one less per B_D^T row)
     for (int32_t z : p->dec.node_zeta) zmax = std::max(zmax, (int)z);
     p->lam_ok = lambda_clusters_ok(p, zmax);
