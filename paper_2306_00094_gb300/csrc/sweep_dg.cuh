@@ -216,19 +216,6 @@ __device__ __forceinline__ double dg_value(long long hi, long long lo, int E) {
     return sign ? -v : v;
 }
 
-// 1 / d for a positive normal d: an FP32 reciprocal of the mantissa and two Newton steps in FP64 (to
-// about an ulp), six FP64 instructions where the division takes some twenty
-__device__ __forceinline__ double dg_recip(double d) {
-    const long long b = __double_as_longlong(d);
-    const int ex = (int)((b >> 52) & 0x7ff);
-    if (b <= 0 || ex < 2 || ex > 2044) return 1.0 / d;
-    const double m = __longlong_as_double((b & 0xfffffffffffffll) | (1023ll << 52));
-    double x = (double)__frcp_rn((float)m);
-    x = __fma_rn(x, __fma_rn(-m, x, 1.0), x);
-    x = __fma_rn(x, __fma_rn(-m, x, 1.0), x);
-    return __longlong_as_double(__double_as_longlong(x) - ((long long)(ex - 1023) << 52));
-}
-
 // invert the pivot block in registers: 544 threads hold the rows of the 4 x 4 blocks (bi, bl <= bi) of
 // the lower triangle; step p needs row p (= column p), kept in shared memory and rewritten by its
 // owners, and the reciprocal of the pivot, which the next pivot's owner forms first, beside the
@@ -269,7 +256,7 @@ __global__ void __launch_bounds__(DG_PIV_THREADS) k_pivot_dg(DigitArgs a) {
             }
     auto pivot = [&](double d, int buf) {
         if (!(d > 0.0)) ok = false;
-        dpiv[buf] = dg_recip(d);
+        dpiv[buf] = 1.0 / d;
     };
     auto publish = [&](int p, int buf) {            // row p of the current matrix
 #pragma unroll
