@@ -178,6 +178,24 @@ def profile_traffic(kernel_src_hash, name="k_apply_tma_peridynamic_2d.md"):
     return val if (val is not None and h == kernel_src_hash) else None
 
 
+def apply_kernel(entry):
+    """Which kernel a tuned shape of the interface apply (a dict of Problem.autotune) runs as: the name
+    its profile and source go by, and the text of the bench line."""
+    what = ("preconditioner S_k apply, FP16 copy" if entry["kind"] == 1
+            else "dense S_k^+ apply, " + ("FP32" if entry["kind"] == 0 else "FP64"))
+    if entry["rc"] == -1:
+        return "apply_mma", ("k_apply_mma (preconditioner S_k apply on the tensor cores: tcgen05 kind::f16, "
+                             "FP16 copy, FP32 accumulators in tensor memory)")
+    # between two column blocks the default, which holds all columns, goes by the smaller block's name
+    unnamed = (entry["rc"] < entry["nrhs"] < 2 * entry["rc"] and (entry["ctas_per_sm"], entry["rows_per_warp"]) == (2, 4)
+               and entry["rc"] < (8 if entry["kind"] == 2 else 16))
+    rc, rows = (2 * entry["rc"], 8 if entry["rc"] == 8 else 4) if unnamed else (entry["rc"], entry["rows_per_warp"])
+    self_refill = rc == 16 and rows == 8 and entry["ctas_per_sm"] == 2
+    return ("apply_self" if self_refill else "apply_tma",
+            f"k_apply_{'self' if self_refill else 'tma'} ({what}; {rc} columns per pass, {entry['ctas_per_sm']} "
+            f"CTAs per SM, {rows} rows per warp)")
+
+
 def kernel_source_hash(name="apply_tma.cuh"):
     with open(os.path.join(ROOT, "paper_2306_00094_gb300", "csrc", name), "rb") as f:
         return hashlib.sha256(f.read()).hexdigest()[:16]
@@ -331,20 +349,18 @@ def run_ours(args):
     hbm, peak_kind = peaks()
     roof = apply_rooflines(torch, prob, step, args.steps, hbm, peak_kind)
     ap, hp = roof["apply"], roof["half_apply"]
+    by_kind = {e["kind"]: e for e in tuned}
+    if args.tensor_core_precond:
+        by_kind[1] = dict(by_kind[1], rc=-1)
+    for roofline, kind in ((ap, 0), (hp, 1)):
+        if roofline:
+            kernel, text = apply_kernel(by_kind[kind])
+            tag = "fp16_" if kind == 1 and kernel != "apply_mma" else ""
+            roofline.update({"kernel": text,
+                             "traffic": profile_traffic(kernel_source_hash(f"{kernel}.cuh"), f"k_{kernel}_{tag}{name}.md")})
     if ap:
-        ap.update({"kernel": "k_apply_tma<float> (dense S_k^+ apply, FP32, tensor-copy pipeline)",
-                   "timing": "CUDA events around each apply launch over a second timed region of the same "
-                             f"{args.steps} steps",
-                   "traffic": profile_traffic(kernel_source_hash(), f"k_apply_tma_{name}.md")})
-    if hp:
-        tc_pre = any(e["kind"] == 1 and e["rc"] == -1 for e in tuned) or args.tensor_core_precond
-        if tc_pre:
-            hp.update({"kernel": "k_apply_mma (preconditioner S_k apply on the tensor cores: tcgen05 kind::f16, "
-                                 "FP16 copy, FP32 accumulators in tensor memory)",
-                       "traffic": profile_traffic(kernel_source_hash("apply_mma.cuh"), f"k_apply_mma_{name}.md")})
-        else:
-            hp.update({"kernel": "k_apply_tma<float, .., __half> (preconditioner S_k apply, FP16 copy)",
-                       "traffic": profile_traffic(kernel_source_hash(), f"k_apply_tma_fp16_{name}.md")})
+        ap["timing"] = ("CUDA events around each apply launch over a second timed region of the same "
+                        f"{args.steps} steps")
 
     # end to end through the C ABI with pinned host buffers
     h_rhs = torch.empty((R, ndof), dtype=torch.float64, pin_memory=True)
