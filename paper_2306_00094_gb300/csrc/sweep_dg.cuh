@@ -199,21 +199,33 @@ template <int W> __device__ __forceinline__ long long dg_lo(const uint32_t (&acc
 // the product sum 2^(E - 16) (hi 2^-27 + lo 2^-54), E the sum of the two rows' exponents, as a double,
 // by integer operations alone (the FP64 pipe takes a warp 64 clocks per instruction; a 64-bit
 // conversion is several): cut to 62 bits, normalised, rounded once to 53 bits (half up) and given
-// exponent and sign
-__device__ __forceinline__ double dg_value(long long hi, long long lo, int E) {
+// exponent and sign.  This form is for the ends of the range and rows that are not finite
+__device__ __forceinline__ double dg_value_ends(long long hi, long long lo, int E) {
     const int sh = min(26, __clzll((hi < 0 ? -hi : hi) | 1) - 2);        // |hi| < 2^48
     const long long I = (hi << sh) + (lo >> (27 - sh));
     const unsigned long long mag = (unsigned long long)(I < 0 ? -I : I);
     const int lz = __clzll(mag | 1);
     const unsigned long long m = mag << lz;                              // leading bit 63
     const long long q = (long long)((m >> 11) + ((m >> 10) & 1));        // 53 bits (or 2^53)
+    if (E >= DG_NAN / 2) return __longlong_as_double(0x7ff8000000000000ll);   // a row was not finite
+    const double v = mag ? ldexp((double)q, E - 43 - sh + 63 - lz - 52) : 0.0;
+    return I < 0 ? -v : v;
+}
+// the same without a branch, where the result is a normal number or zero; elsewhere ends is set.  The
+// lanes stay together: the loads of the accumulators are .aligned, and bringing the warp together
+// before each cost k_update_dg 118 of 578 us (6 x 6 table row, a step's average)
+__device__ __forceinline__ double dg_value(long long hi, long long lo, int E, bool &ends) {
+    const int sh = min(26, __clzll((hi < 0 ? -hi : hi) | 1) - 2);
+    const long long I = (hi << sh) + (lo >> (27 - sh));
+    const unsigned long long mag = (unsigned long long)(I < 0 ? -I : I);
+    const int lz = __clzll(mag | 1);
+    const unsigned long long m = mag << lz;
+    const long long q = (long long)((m >> 11) + ((m >> 10) & 1));
     // value q 2^(e - 52), e the exponent of the leading bit
     const int e = E - 43 - sh + 63 - lz;
-    const long long sign = I < 0 ? (1ll << 63) : 0;
-    if (mag != 0 && e > -1022 && e < 1023) return __longlong_as_double((q + ((long long)(e + 1022) << 52)) | sign);
-    if (E >= DG_NAN / 2) return __longlong_as_double(0x7ff8000000000000ll);   // a row was not finite
-    const double v = mag ? ldexp((double)q, e - 52) : 0.0;
-    return sign ? -v : v;
+    ends |= (mag != 0 && (e <= -1022 || e >= 1023)) || E >= DG_NAN / 2;
+    const long long b = (q + ((long long)(e + 1022) << 52)) | (I < 0 ? (1ll << 63) : 0);
+    return __longlong_as_double(mag != 0 ? b : 0ll);
 }
 
 // invert the pivot block in registers: 544 threads hold the rows of the 4 x 4 blocks (bi, bl <= bi) of
@@ -426,8 +438,7 @@ __global__ void __launch_bounds__(DG_PAN_THREADS, 1) k_panel_dg(DigitArgs a) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     // (scaled) pan = old D^-1: lane quarter warp mod 4 and columns 16 (warp / 4) .. are the thread's own
 #pragma unroll
-    for (int c0 = 0; c0 < 16; c0 += 8) {
-        __syncwarp();                                // dg_value branches; the loads are .aligned
+    for (int c0 = 0; c0 < 16; c0 += 8) {               // the lanes part only where __syncwarp() follows
         uint32_t hi[DG_HI][8], lo[DG - DG_HI][8];
         const uint32_t ta = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(16 * h + c0);
 #pragma unroll
@@ -435,9 +446,16 @@ __global__ void __launch_bounds__(DG_PAN_THREADS, 1) k_panel_dg(DigitArgs a) {
 #pragma unroll
         for (int d = DG_HI; d < DG; ++d) dg_ld8(ta + (uint32_t)(d * NB), lo[d - DG_HI]);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        bool ends = false;
 #pragma unroll
         for (int c = 0; c < 8; ++c)
-            x[c0 + c] = dg_value(dg_hi(hi, c), dg_lo(lo, c), Eo + sde[16 * h + c0 + c]);
+            x[c0 + c] = dg_value(dg_hi(hi, c), dg_lo(lo, c), Eo + sde[16 * h + c0 + c], ends);
+        if (__any_sync(0xffffffffu, ends)) {
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                x[c0 + c] = dg_value_ends(dg_hi(hi, c), dg_lo(lo, c), Eo + sde[16 * h + c0 + c]);
+            __syncwarp();
+        }
     }
     __syncthreads();                                 // se is written again
     const int Ep = row_exp();
@@ -623,8 +641,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_update_dg(DigitArgs a) {
             }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-            for (int cc = 0; cc < 16; cc += 4) {
-                __syncwarp();                        // dg_value and the stores branch
+            for (int cc = 0; cc < 16; cc += 4) {       // the lanes part only where __syncwarp() follows
                 uint32_t acc[DG - DG_HI][4];
 #pragma unroll
                 for (int d = DG_HI; d < DG; ++d) dg_ld4(ta + (uint32_t)(d * DG_LB + cc), acc[d - DG_HI]);
@@ -635,12 +652,25 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_update_dg(DigitArgs a) {
                     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                     dg_bar_arrive(&acc_empty[1]);
                 }
+                double o[4];
+                bool ends = false;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const double o = m[cc + c] - dg_value(hi[cc + c], dg_lo(acc, c), Ea + eo[c]);
-                    const int l = l0 + cc + c;       // J holds its new values already
-                    if (plain || (in && !iJ && l < n && (l < j0 || l >= j1)))
-                        Mp[(int64_t)(cc + c) * ld] = o;
+                for (int c = 0; c < 4; ++c) o[c] = dg_value(hi[cc + c], dg_lo(acc, c), Ea + eo[c], ends);
+                if (__any_sync(0xffffffffu, ends)) {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) o[c] = dg_value_ends(hi[cc + c], dg_lo(acc, c), Ea + eo[c]);
+                    __syncwarp();
+                }
+                if (plain) {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) Mp[(int64_t)(cc + c) * ld] = m[cc + c] - o[c];
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const int l = l0 + cc + c;   // J holds its new values already
+                        if (in && !iJ && l < n && (l < j0 || l >= j1)) Mp[(int64_t)(cc + c) * ld] = m[cc + c] - o[c];
+                    }
+                    __syncwarp();
                 }
             }
         }

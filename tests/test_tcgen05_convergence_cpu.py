@@ -3,9 +3,9 @@
 ``.sync.aligned`` forms need every thread of the warp at the same instruction, and the compiler need
 not bring a warp together after a branch that its lanes took differently.  So a ``__syncwarp()``
 stands between any such branch and the next aligned instruction: before every deallocation of tensor
-memory (one lane's copies and waits lie before it) and at the head of every loop whose passes load
-accumulators and then store per lane.  Read from the sources: an unconverged warp at such an
-instruction is undefined, so this is not found out by running it.
+memory (one lane's copies and waits lie before it), and in every loop whose passes load accumulators
+and then branch per lane.  Read from the sources: an unconverged warp at such an instruction is
+undefined, so this is not found out by running it.
 """
 import glob
 import os
@@ -40,8 +40,22 @@ def test_deallocation_by_a_converged_warp(name, line):
 @pytest.mark.parametrize("name,line", [(n, i) for n, i in _uses(LOADS.pattern)
                                        if "__device__" not in dict(_lines())[n][i]])
 def test_loads_in_a_loop_by_a_converged_warp(name, line):
-    """Back from the load to the head of its loop over accumulator columns (cc or c0)."""
+    """The pass of the loop over accumulator columns (cc or c0) that holds the load: the warp is brought
+    together before the load, or where its lanes part later in the pass."""
     lines = dict(_lines())[name]
     head = next(i for i in range(line, -1, -1) if re.search(r"for \(int (cc|c0) = 0;", lines[i]))
     assert line - head < 12, f"{name}:{line + 1}: no loop over accumulator columns"
-    assert any("__syncwarp();" in ln for ln in lines[head:line]), f"{name}:{line + 1}"
+    depth, body = 0, []
+    for ln in lines[head:]:
+        depth += ln.count("{") - ln.count("}")
+        body.append(ln)
+        if depth == 0:
+            break
+    if any("__syncwarp();" in ln for ln in body[:line - head]):
+        return
+    # blocks entered by some lanes alone end with the warp brought together
+    parts = [i for i, ln in enumerate(body) if "if (__any_sync(" in ln or "} else {" in ln]
+    assert parts, f"{name}:{line + 1}"
+    for i in parts:
+        close = next(k for k in range(i + 1, len(body)) if body[k].rstrip() == " " * (len(body[i]) - len(body[i].lstrip())) + "}")
+        assert body[close - 1].strip() == "__syncwarp();", f"{name}:{head + close}"
