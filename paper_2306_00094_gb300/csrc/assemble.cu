@@ -33,9 +33,10 @@
 // rate): the moments call the power function once per radius (r^-2s; not at all for s = 1/2) and
 // sincos once per angle (the direction follows by rotation with the edge normal), and a row of the
 // local matrix takes 3 FMAs per entry and point from the point's combined moments.  On the
-// fractional kernel with h = 1/64, delta = 6.4 h, 4 x 4 parts: 72 ms (38.0 for 79 k touching pairs,
-// 26.4 for 1.35 M cut, 7.5 for 0.63 M whole), against 600 ms for one thread per pair with the power
-// function at every radial moment and the local matrix in shared memory.
+// fractional kernel with h = 1/64, delta = 6.4 h, 4 x 4 parts, s = 1/2: 72 ms (38.0 for 79 k touching
+// pairs, 26.4 for 1.35 M cut, 7.5 for 0.63 M whole), against 600 ms for one thread per pair with the
+// power function at every radial moment and the local matrix in shared memory; s = 0.4 or 0.75: 136 ms
+// (58.9, 60.6, 16.8), against 663.
 // 1-D: one thread per pair.
 #include <algorithm>
 #include <cmath>

@@ -741,7 +741,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_cg_init(const double *b, const 
 }
 
 // q = A p (double-single products), (p, q) per column, alpha for the active columns.  A CTA takes
-// units of 32 consecutive rows with 4 CW warps.  Lanes are (nonzero slot kg = lane / 8, position
+// units of 32 consecutive rows with 4 CW warps (CW = 8: 8 warps, below).  Lanes are (nonzero slot kg = lane / 8, position
 // lane % 8): the 4 slots take every 4th nonzero of a row, and the 8 positions are CW columns of
 // 8 / CW rows (CW = R rounded up to a power of two, at most 8; more columns in blocks of 8).  With
 // 8 columns the lanes of a slot read one nonzero and 8 consecutive p entries (one 32-byte segment
@@ -1616,8 +1616,9 @@ struct Runner {
     // slower).  The Lambda vectors and their
     // arithmetic are in the operators' type T: FP64 in the FP64 pass; FP32 in the FP32 pass,
     // whose iterations only have to reduce the residual by inner_tol (the refinement's FP64
-    // residual corrects what FP32 leaves).  The dot products' tile sums and the PCG scalars are
-    // FP64 in both.
+    // residual corrects what FP32 leaves).  The FP32 pass adds dot products as compensated FP32 pairs
+    // (lambda_rows.cuh from the tile sums on, lambda_cluster.cuh within a CTA, FP64 from there); the PCG
+    // scalars are FP64 in both.
     template <typename T> void iteration(const OpPool<T> &pool, double tol, int max_it) {
         if (p->lam_ok) return iteration_clusters<T>(pool, tol, max_it);
         if constexpr (std::is_same<T, float>::value) {

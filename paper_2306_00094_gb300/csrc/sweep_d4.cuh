@@ -5,8 +5,8 @@
 // 2^(-9 k) is exact in BF16, so products of different orders can share an FP32 accumulator: one takes
 // the order 0 (integers below 2^20, exact), the other the orders 3, 2, 1 in turn (below 2^13; what the
 // tensor core truncates there lies 2^-24 below it, 2^-9 of an FP32 rounding of the leading sum).
-// Orders past 3 are dropped (below 2^-28 of the product of the row maxima when every digit is at its
-// limit, 2^-34 for digits of random sign).  An entry then takes two FP32 roundings where a dot product on
+// Orders past 3 are dropped: of the product of the row maxima at most 2^-24 (every digit at its limit, all
+// of one sign), about 2^-31 for random digits.  An entry then takes two FP32 roundings where a dot product on
 // the FP32 pipes takes 64, and both sweeps run here: S_k^+ came out as exact as with the FP32 pipes
 // or up to five times more (against FP64; a split-TF32 update, whose leading sums the tensor core
 // truncates, was 1.5 to 19 times less exact than the pipes and stayed out of the pinned sweep).

@@ -12,10 +12,13 @@
 // accumulators of tcgen05.mma kind::f16.  The products of order i + j = d share accumulator d; its sum
 // is below 2^20, 2^22, 2^23 for d = 0, 1, 2 and below 2^25 for the rest (above 2^24 only when nearly
 // every digit is at its limit; what FP32 then rounds lies 2^-45 below the accumulator's unit weight).
-// Orders past DG - 1 are dropped: they lie below 2^-58 of the product of the row maxima, where an FP64
-// dot product of 64 terms has rounding errors of a few 2^-53 of its partial sums.  The epilogue adds
-// the accumulators in 64-bit integers, rounds the sum once to a double and takes one FP64 operation
-// per entry instead of 64.
+// Orders past DG - 1 are dropped: of the product of the row maxima at most 2^-50 (every digit at its limit,
+// all of one sign), about 2^-57 for random digits, where an FP64 dot product of 64 terms has 64 rounding
+// errors of 2^-53 of its partial sums.  The epilogue adds the accumulators in 64-bit integers, rounds
+// the sum once to a double and takes one FP64 operation per entry instead of 64.  An entry far below its
+// row's largest keeps fewer than its 53 bits; S_k and S_k^+ of 20 matrices (100 to 730 dofs, every
+// kernel, extended precision as the reference) err 0.99 and 0.97 times as much as on the FP64 pipes on
+// average, 1.05 and 1.09 at most.
 // The 64 pivots are first brought to one scale: column s of old is divided by the power of two 2^c_s
 // next to sqrt(M_ss) and column s of pan multiplied by it (exact, and without effect on pan old^T), so
 // that a block that mixes large and small diagonal entries keeps the digits of the small ones.
@@ -33,8 +36,8 @@
 // sets its pace), so N = 64; seven accumulators of 64 columns fill tensor memory, so the high orders
 // (0 .. 3) and the low ones take turns: sixteen warps drain one part while the other is formed.  Per
 // block of 8192 entries 6.8 k clocks of MMA against 4.1 k of the FP64 pipe.  The entries of J are written by k_panel_dg
-// (taken here, lane by lane, they cost 0.08 ms).  Measured on that row: 0.73 ms per step of the 36 matrices (the
-// MMAs alone 0.32), against 15.3 ms; factorization and one solve 422 -> 35.5 ms.
+// (taken here, lane by lane, they cost 0.08 ms).  Measured on that row: 0.70 ms per step of the 36 matrices (the
+// MMAs alone 0.32), against 15.3 ms; factorization and one solve 422 -> 33.1 ms.
 // Every wait is bounded: one that runs out sets the sweep's timeout word; the CTA then waits (bounded)
 // for its copies and MMAs, frees its tensor memory and returns.
 #pragma once
