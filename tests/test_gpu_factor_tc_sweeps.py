@@ -3,7 +3,6 @@
 Read from the kernels of a factorization; and where a sweep is the same, so are its bits: S_k comes
 from the Omega sweep alone, S_k^+ from both.
 """
-import json
 import os
 import sys
 
@@ -29,7 +28,7 @@ def _measure():
         p.set_options(binding.default_options(precision=1, **({} if tc == "default" else {"factor_tc": tc})))
         got = names(lambda: p.factor(2), "k_update")
         out[str(tc)] = sorted({"digits" if "k_update_d4" in n else "pipes" for n in got})
-    print(json.dumps(out))
+    return out
 
 
 def test_the_sweeps_of_each_setting():
@@ -53,4 +52,5 @@ def test_the_operators_of_each_setting():
 
 if __name__ == "__main__":
     sys.path.insert(0, os.path.dirname(os.path.abspath(__file__)))
-    _measure()
+    import kernel_names
+    kernel_names.main(_measure)
